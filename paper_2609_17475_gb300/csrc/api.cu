@@ -28,11 +28,9 @@ int launch_tq4_decode(const Geom&, const jf_kv_pool&, const CUtensorMap&, const 
                       float, void*, void*, int32_t, cudaStream_t, const void*, const void*,
                       int32_t);
 int decode_box_rows();
-int launch_prefill(const Geom&, const jf_kv_pool&, const CUtensorMap&, const int32_t*,
-                   const void*, int32_t, int32_t, int32_t, float, int32_t, void*, void*,
-                   cudaStream_t);
-int launch_prefill_batch(const Geom&, const jf_kv_pool&, const int32_t* const*, const int32_t*,
-                         const int32_t*, const void*, const int64_t*, int32_t, int32_t, float,
+int prefill_box_rows(bool v);
+int launch_prefill_batch(const Geom&, const jf_kv_pool&, const CUtensorMap*,
+                         const int32_t* const*, const int32_t*, const int32_t*, const void*, const int64_t*, int32_t, int32_t, float,
                          int32_t, void*, void*, cudaStream_t, int32_t, int64_t,
                          const Tq4Params*);
 size_t prefill_workspace_bytes(int64_t rows, int64_t Hq, int64_t D, int64_t S, int fmt);
@@ -93,21 +91,31 @@ EncodeTiledFn encode_fn() {
 }
 
 // 5-D map over the code rows of a pool: (byte in row, slot, KV head, K|V, page),
-// box = (row bytes, rows_per_box, 1, 1, 1), 128B (or 64B) swizzle.
-int make_codes_map(const Geom& g, void* base, int rows_per_box, CUtensorMap* map) {
+// box = (row_bytes, rows_per_box, 1, 1, 1), swizzled over its row (128, 64 or
+// 32 bytes; 16-byte rows are not swizzled).
+int make_codes_map(const Geom& g, void* base, int row_bytes, int rows_per_box, CUtensorMap* map) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return JF_ERR_CUDA;
   cuuint64_t dims[5] = {(cuuint64_t)g.CB, (cuuint64_t)g.P, (cuuint64_t)g.Hkv, 2,
                         (cuuint64_t)g.num_pages};
   cuuint64_t strides[4] = {(cuuint64_t)g.CB, (cuuint64_t)g.P * g.CB,
                            (cuuint64_t)g.codes_region, (cuuint64_t)g.page_bytes};
-  cuuint32_t box[5] = {(cuuint32_t)g.CB, (cuuint32_t)rows_per_box, 1, 1, 1};
+  cuuint32_t box[5] = {(cuuint32_t)row_bytes, (cuuint32_t)rows_per_box, 1, 1, 1};
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  CUtensorMapSwizzle sw = g.CB == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+  CUtensorMapSwizzle sw = row_bytes == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
+                          : row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                          : row_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                            : CU_TENSOR_MAP_SWIZZLE_NONE;
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, base, dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? JF_OK : JF_ERR_CUDA;
+}
+
+// The prefill kernel's K and V boxes.
+int make_prefill_maps(const Geom& g, void* base, CUtensorMap (&maps)[2]) {
+  const int st = make_codes_map(g, base, g.CB, prefill_box_rows(false), &maps[0]);
+  return st ? st : make_codes_map(g, base, g.CB / 2, prefill_box_rows(true), &maps[1]);
 }
 
 }  // namespace
@@ -200,7 +208,7 @@ static int decode_common(const jf_kv_pool* pool, const int32_t* page_table, int3
     if (st) return st;
   }
   CUtensorMap tmap;
-  st = make_codes_map(g, pool->base, decode_box_rows(), &tmap);
+  st = make_codes_map(g, pool->base, g.CB, decode_box_rows(), &tmap);
   if (st) return st;
   if (pool->format == JF_FMT_TQ4) {
     return launch_tq4_decode(g, *pool, tmap, prm, page_table, pt_stride, context_lens, batch, q,
@@ -351,6 +359,9 @@ int jf_prefill_chunk_attn(const jf_kv_pool* pool, const int32_t* page_table_row,
     st = tq4_make_params(pool->tq4, g.D, &prm);
     if (st) return st;
   }
+  CUtensorMap maps[2];
+  st = make_prefill_maps(g, pool->base, maps);
+  if (st) return st;
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int64_t row0 = 0;
   const PfTailPlan p = prefill_tail_plan(num_q_heads / pool->num_kv_heads, pool->num_kv_heads,
@@ -362,21 +373,17 @@ int jf_prefill_chunk_attn(const jf_kv_pool* pool, const int32_t* page_table_row,
     const int32_t t_start = q_start + p.head, t_len = chunk_len - p.head;
     const void* q_t = static_cast<const uint8_t*>(q) + (size_t)p.head * row_bytes;
     void* out_t = static_cast<uint8_t*>(out) + (size_t)p.head * row_bytes;
-    st = launch_prefill_batch(g, *pool, &page_table_row, &q_start, &p.head, q, &row0, 1,
+    st = launch_prefill_batch(g, *pool, maps, &page_table_row, &q_start, &p.head, q, &row0, 1,
                               num_q_heads, softmax_scale, causal, out, workspace, s, 1, p.head,
                               tq ? &prm : nullptr);
     if (st) return st;
-    return launch_prefill_batch(g, *pool, &page_table_row, &t_start, &t_len, q_t, &row0, 1,
+    return launch_prefill_batch(g, *pool, maps, &page_table_row, &t_start, &t_len, q_t, &row0, 1,
                                 num_q_heads, softmax_scale, causal, out_t, workspace, s, p.k,
                                 t_len, tq ? &prm : nullptr);
   }
-  if (tq)
-    return launch_prefill_batch(g, *pool, &page_table_row, &q_start, &chunk_len, q, &row0, 1,
-                                num_q_heads, softmax_scale, causal, out, workspace, s, 1,
-                                chunk_len, &prm);
-  CUtensorMap tmap{};
-  return launch_prefill(g, *pool, tmap, page_table_row, q, q_start, chunk_len, num_q_heads,
-                        softmax_scale, causal, out, workspace, s);
+  return launch_prefill_batch(g, *pool, maps, &page_table_row, &q_start, &chunk_len, q, &row0, 1,
+                              num_q_heads, softmax_scale, causal, out, workspace, s, 1, chunk_len,
+                              tq ? &prm : nullptr);
 }
 
 size_t jf_prefill_batch_workspace_bytes(int32_t format, int64_t total_rows, int32_t num_q_heads,
@@ -424,7 +431,10 @@ int jf_prefill_batch_attn(const jf_kv_pool* pool, const int32_t* page_table, int
     st = tq4_make_params(pool->tq4, g.D, &prm);
     if (st) return st;
   }
-  return launch_prefill_batch(g, *pool, rows, q_start, chunk_len, q, row0, batch, num_q_heads,
+  CUtensorMap maps[2];
+  st = make_prefill_maps(g, pool->base, maps);
+  if (st) return st;
+  return launch_prefill_batch(g, *pool, maps, rows, q_start, chunk_len, q, row0, batch, num_q_heads,
                               softmax_scale, causal, out, workspace,
                               static_cast<cudaStream_t>(stream), num_splits, acc,
                               pool->format == JF_FMT_TQ4 ? &prm : nullptr);
@@ -522,7 +532,7 @@ int jf_paged_decode_attn_noalloc(const jf_kv_pool* pool, const int32_t* page_tab
   if (cudaMemsetAsync(ws, 0, sizeof(int32_t), s) != cudaSuccess) return JF_ERR_CUDA;
   const Geom g = make_geom(*pool);
   CUtensorMap tmap;
-  st = make_codes_map(g, pool->base, decode_box_rows(), &tmap);
+  st = make_codes_map(g, pool->base, g.CB, decode_box_rows(), &tmap);
   if (st) return st;
   st = launch_decode(g, *pool, tmap, page_table, pt_stride, context_lens, batch, q, num_q_heads,
                      softmax_scale, out, ws, num_splits, s);

@@ -18,8 +18,12 @@
 // D/2 of the V columns (its N half of O += P V) -- so the dequantization work
 // per SM is halved while each SM's tensor core still does its 128 rows.
 // Warp roles (each CTA):
-//   warp 0      TMEM allocation (512 columns, pair-wide); in CTA 0, lane 0
-//               issues every tcgen05.mma.cta_group::2 of the pair:
+//   warp 0      TMEM allocation (512 columns, pair-wide); in CTA 0 it issues
+//               every tcgen05.mma.cta_group::2 of the pair.  The whole warp
+//               runs the issuing code and an elected lane issues, so that
+//               descriptors and addresses stay in uniform registers: issued
+//               from a branch of one lane, the 16 MMAs of one S took ~1,470
+//               cycles to issue for 1,024 of tensor work; now ~120.
 //                 S_i  = Q  [K_2i K_2i+1]^T  (A = Q in smem, B = the K halves
 //                        of tiles 2i and 2i + 1 in smem, K-major, N = 128)
 //                 O   += P_j V_j             (A = P_j in TMEM, B = V_j smem,
@@ -29,13 +33,12 @@
 //               [D, D + 256); P_j (fp16) overwrites S columns already read.
 //               S over two tiles keeps the MMA at N = 128 (an N = 64 pair
 //               MMA takes as long as an N = 128 one).
-//   warps 1-8   dequantize this CTA's halves of 64-position K/V tiles from
-//               the pool (page-table lookup, 4-bit codes -> fp16 integers
-//               through the mantissa of fp16 1024, then x = code * scale +
-//               bias with one fused multiply-add) into 128B-swizzled
-//               buffers, one item (one position's code bytes of a 64-wide
-//               block) per thread, loads running two tiles ahead; warps 1-4
-//               write K halves into two pair buffers (free again once S of
+//   warps 1-8   dequantize this CTA's halves of 64-position K/V tiles
+//               (4-bit codes -> fp16 integers through the mantissa of fp16
+//               1024, then x = code * scale + bias with one fused
+//               multiply-add) into 128B-swizzled buffers, one item (one
+//               position's code bytes of a 64-wide block) per thread; warps
+//               1-4 write K halves into two pair buffers (free again once S of
 //               the pair two back is done), warps 5-8 V halves into four
 //               tile buffers (free once P V of the tile four back is done),
 //               each arriving on CTA 0's K-pair or V-tile barrier.
@@ -45,6 +48,20 @@
 //               CTA 0's P barrier; the running maximum is moved only when it
 //               grows by more than 2^8, and then O is rescaled in TMEM;
 //               finally O / l -> bf16 output.
+//   warp 13     one lane copies the packed codes and side words of the tiles
+//               ahead from the pool into a ring of NST stages by TMA (it also
+//               looks the pages up).  The dequantization warps, the slowest
+//               link of the chain, then touch no global memory and no
+//               addresses: with their own loads (a tag lookup for each
+//               position and 16 bytes, ~770 cycles of the SM's load path a
+//               tile, divisions for the page and slot) a K tile took them
+//               ~2,400 cycles, now ~1,800.  A warp of its own, because the
+//               dequantization warps' proxy fences wait for copies that they
+//               issued themselves (2,048 queries after 30,720 positions: 1,848
+//               us with the copies issued by each of those warps, 1,528 us from
+//               here).  With the two changes above that case went from 1,525
+//               to 1,196 us, 8 chunks of 64 queries after 4K-32K positions from
+//               354 to 269 us.
 // Within every 8 consecutive d the tiles store elements in the order
 // 0,4,1,5,2,6,3,7 (the pairs one 32-bit word of codes yields); Q uses the same
 // order, so Q K^T is unchanged, and the epilogue undoes it for O.  Q is
@@ -61,7 +78,8 @@ constexpr int PF_BM = 128;   // MMA rows per CTA (256 per CTA pair)
 constexpr int PF_BN = 64;    // positions per K/V tile
 constexpr int PF_DQ_WARPS = 8;
 constexpr int PF_SM_WARPS = 4;   // one per TMEM lane quarter, one row per thread
-constexpr int PF_THREADS = 32 * (1 + PF_DQ_WARPS + PF_SM_WARPS);
+constexpr int PF_THREADS = 32 * (2 + PF_DQ_WARPS + PF_SM_WARPS);
+constexpr int PF_TMA_WARP = 1 + PF_DQ_WARPS + PF_SM_WARPS;   // the code copies' producer
 constexpr int PF_KVBUF = 4;     // P V completion barriers, by tile index mod 4
 constexpr float PF_TAU = 8.f;   // log2 headroom before the running max moves
 
@@ -84,7 +102,7 @@ struct PrefillArgs {
   int64_t codes_region;
   int64_t sb_base;
   int64_t sb_region;
-  int32_t P, Hkv, Hq, G, QPC;
+  int32_t P, log2P, Hkv, Hq, G, QPC;   // P is a power of two
   int32_t causal;
   float scale_log2;
   int32_t* status;
@@ -104,16 +122,27 @@ struct PrefillArgs {
 // (rows 32 (j & 1) + t), so one N = 128 MMA computes S for both.
 template <int D, int FMT>
 struct PfSmem {
-  static constexpr int VB = 4;                           // V tile buffers
+  static constexpr bool TQ = FMT == JF_FMT_TQ4;
+  // V tile buffers, and tiles of packed codes in flight: what is left of the
+  // 227 KB (TQ4 at D = 256 gives up a V buffer, its centroid table holding
+  // 32 KB)
+  static constexpr int VB = (TQ && D == 256) ? 3 : 4;
+  static constexpr int NST = (TQ && D == 256) ? 2 : 3;
+  static constexpr int BOX_BYTES = 16 * D;   // this CTA's codes of a tile: K half, or V half
+  static constexpr int SBB = TQ ? 2 : D / 16;                // side bytes of a vector
+  static constexpr int SIDE_BYTES = (PF_BN / 2 + PF_BN) * SBB;   // K half's, then V's
+  static constexpr uint32_t STAGE_TX = 2 * BOX_BYTES + SIDE_BYTES;
   static constexpr int Q_BYTES = PF_BM * D * 2;          // [D/64][128 rows][128 B]
   static constexpr int KP_BYTES = PF_BN * D * 2;         // [D/64][64 rows][128 B]
   static constexpr int VT_BYTES = PF_BN * (D / 2) * 2;   // [D/128][64 rows][128 B]
   static constexpr int OFF_Q = 0;
   static constexpr int OFF_K = Q_BYTES;
   static constexpr int OFF_V = OFF_K + 2 * KP_BYTES;
-  static constexpr int OFF_BAR = OFF_V + VB * VT_BYTES;
+  static constexpr int OFF_STG = OFF_V + VB * VT_BYTES;   // code stages [NST][K | V]
+  static constexpr int OFF_SIDE = OFF_STG + NST * 2 * BOX_BYTES;   // side words [NST]
+  static constexpr int OFF_BAR = OFF_SIDE + NST * SIDE_BYTES;
   static constexpr int OFF_LUT = OFF_BAR + 256;   // TQ4 centroid table (lane-replicated)
-  static constexpr int TOTAL = 1024 + OFF_LUT + (FMT == JF_FMT_TQ4 ? 256 * 32 * 4 : 0);
+  static constexpr int TOTAL = 1024 + OFF_LUT + (TQ ? 256 * 32 * 4 : 0);
   static_assert(TOTAL <= 227 * 1024, "shared memory per CTA");
 };
 
@@ -185,12 +214,12 @@ __device__ __forceinline__ void sb_to_h2(uint32_t w, uint32_t& s2, uint32_t& b2)
 // natural d order, partial outputs rotated back by the merge kernel)
 template <int D, int FMT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
-prefill_kernel(const __grid_constant__ PrefillArgs a) {
+prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
+               const __grid_constant__ PrefillArgs a) {
   using L = PfSmem<D, FMT>;
   constexpr bool TQ = FMT == JF_FMT_TQ4;
   constexpr int NKB = D / 64;           // 64-wide d blocks
   constexpr int UPI = (D == 256) ? 2 : 1;   // 16-byte code units per dequant item
-  constexpr int SBB = D / 16;
   constexpr int CB = D / 2;
   // 128 K items (32 positions x NKB blocks x 2/UPI units) + 128 V items
   // (64 positions x NKB/2 blocks x 2/UPI units): one per dequant thread
@@ -216,8 +245,11 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
   // out of the phase the other CTA has not reached.
   uint64_t* p_full = bars + 12;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
+  uint64_t* stg_full = bars + 18;                // [NST] a tile's code bytes have landed
+  uint64_t* stg_free = bars + 18 + L::NST;       // [NST] ... and have been read
+  int32_t* stg_ok = reinterpret_cast<int32_t*>(bars + 18 + 2 * L::NST);   // [NST] page id was valid
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_rank();
   // CTA pairs in launch order: the KV heads of one pair of query tiles are
   // consecutive, so every head's longest tiles start in the first wave
@@ -264,7 +296,13 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
       mbar_init(&k_full[i], 2 * PF_DQ_WARPS);    // the 4 K warps of each CTA, twice
       mbar_init(&s_full[i], 1);
     }
+    for (int i = 0; i < L::NST; ++i) {
+      mbar_init(&stg_full[i], 1);
+      mbar_init(&stg_free[i], PF_DQ_WARPS);
+    }
     fence_barrier_init();
+    prefetch_tensormap(&kmap);
+    prefetch_tensormap(&vmap);
   }
   if constexpr (TQ) {   // centroid pair of code byte b for lane l: word b * 32 + l
     uint32_t* lut = reinterpret_cast<uint32_t*>(sm + L::OFF_LUT);
@@ -276,7 +314,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
   __syncthreads();
   tc::cluster_sync();   // both CTAs: barriers initialized, TMEM allocated
   tc::fence_after();
-  const uint32_t tbase = *tmem_slot;
+  const uint32_t tbase = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const uint32_t tO = tbase;
   const uint32_t tS = tbase + D;               // two S/P buffers of 2 PF_BN columns
 
@@ -294,7 +332,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
     return reinterpret_cast<uint4*>(sQ + (m >> 3) * (PF_BM * 128) + r * 128 +
                                     (((m & 7) ^ (r & 7)) << 4));
   };
-  if (TQ && warp > PF_DQ_WARPS) {
+  if (TQ && warp > PF_DQ_WARPS && warp < PF_TMA_WARP) {
     // rotated fp32 query row, natural d order (the centroid pairs are too)
     const float* qrow = a.qrot + ((int64_t)(rq.row0 + q0 + qi) * a.Hq + kvh * a.G + r % a.G) * D;
     float qmax = 0.f;
@@ -318,7 +356,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
                                pack_f16x2(w1.x * qs, w1.y * qs), pack_f16x2(w1.z * qs, w1.w * qs));
     }
     fence_proxy_async_smem();
-  } else if (warp > PF_DQ_WARPS) {
+  } else if (warp > PF_DQ_WARPS && warp < PF_TMA_WARP) {
     const uint16_t* qrow = rq.q + ((int64_t)(q0 + qi) * a.Hq + kvh * a.G + r % a.G) * D;
     float qmax = 0.f;
     if (row_ok) {
@@ -353,8 +391,11 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
 
   if (warp == 0) {
     // ================= MMA issuer (CTA 0 of the pair) =================
-    if (rank == 0 && lane == 0) {
-      const uint32_t qaddr = smem_u32(sQ), kaddr = smem_u32(sK), vaddr = smem_u32(sV);
+    if (rank == 0) {
+      const uint32_t leader = tc::elect_one();
+      const uint64_t qdesc = tc::sdesc_sw128(smem_u32(sQ), 16, 1024);
+      const uint64_t kdesc = tc::sdesc_sw128(smem_u32(sK), 16, 1024);
+      const uint64_t vdesc = tc::sdesc_sw128(smem_u32(sV), PF_BN * 128, 1024);
       bool ok = true;
       // P_j (fp16, 32 columns) sits in the columns of its pair's S buffer
       // that held S of positions 0..31 of tile j
@@ -366,10 +407,9 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
         const uint32_t tp = tS + ((j >> 1) & 1) * (2 * PF_BN) + (j & 1) * 32;
 #pragma unroll
         for (int k = 0; k < PF_BN / 16; ++k)
-          tc::mma2_ts(tO, tp + 8 * k,
-                      tc::sdesc_sw128(vaddr + kb * L::VT_BYTES + k * 2048, PF_BN * 128, 1024),
-                      IDPV, (j > 0 || k > 0) ? 1u : 0u);
-        tc::commit2_both(&pv_done[j & 3]);
+          tc::mma2_ts(leader, tO, tp + 8 * k, vdesc + ((kb * L::VT_BYTES + k * 2048) >> 4), IDPV,
+                      (j > 0 || k > 0) ? 1u : 0u);
+        tc::commit2_both(leader, &pv_done[j & 3]);
       };
       // Pair i: S of tiles 2i, 2i + 1 into S buffer i & 1 (S column n = K row
       // n of CTA 0 for n < 64, row n - 64 of CTA 1 otherwise: position 32 rank
@@ -385,74 +425,58 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
           tc::fence_after();
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma2_ss(tS + (i & 1) * (2 * PF_BN),
-                        tc::sdesc_sw128(qaddr + (ks >> 2) * (PF_BM * 128) + (ks & 3) * 32, 16, 1024),
-                        tc::sdesc_sw128(kaddr + (i & 1) * L::KP_BYTES + (ks >> 2) * (PF_BN * 128) +
-                                            (ks & 3) * 32, 16, 1024),
+            tc::mma2_ss(leader, tS + (i & 1) * (2 * PF_BN),
+                        qdesc + (((ks >> 2) * (PF_BM * 128) + (ks & 3) * 32) >> 4),
+                        kdesc + (((i & 1) * L::KP_BYTES + (ks >> 2) * (PF_BN * 128) +
+                                  (ks & 3) * 32) >> 4),
                         IDQK, ks ? 1u : 0u);
-          tc::commit2_both(&s_full[i & 1]);
+          tc::commit2_both(leader, &s_full[i & 1]);
         }
         for (const int upto = i < npairs ? 2 * i : ntiles; jn < upto && ok; ++jn) pv(jn);
       }
-      if (!ok) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
+      if (!ok && lane == 0) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
     }
     __syncwarp();
   } else if (warp <= PF_DQ_WARPS) {
     // ================= dequantization (this CTA's halves) =================
-    // threads 0..127: K item (position 32 rank + t of the tile, block kb, unit u0)
-    // threads 128..255: V item (position t, block D/128 * rank + kbl, unit u0)
+    // One item per thread: the code bytes of one position, 16 UPI of them.
+    // K warp w: positions 32 rank + 8 w .. + 7 of the tile, whole rows (4 items
+    // each); V warp w: positions 16 w .. + 15, this CTA's half rows (2 items).
     const int dt = (int)threadIdx.x - 32;
     const bool is_v = dt >= 128;
-    const int e = is_v ? dt - 128 : dt;
-    const int t = is_v ? (e % PF_BN) : (e % (PF_BN / 2));
-    const int rest = is_v ? (e / PF_BN) : (e / (PF_BN / 2));
-    const int kbl = (UPI == 2) ? rest : (is_v ? 0 : rest >> 1);
-    const int u0 = (UPI == 2) ? 0 : (is_v ? rest : rest & 1);
+    const int dw = (warp - 1) & 3;
+    const int t = is_v ? 16 * dw + (lane & 15) : 8 * dw + (lane & 7);
+    const int unit = is_v ? lane >> 4 : lane >> 3;
+    const int kbl = (UPI == 2) ? unit : unit >> 1;
+    const int u0 = (UPI == 2) ? 0 : unit & 1;
     const int kb = is_v ? (NKB / 2) * (int)rank + kbl : kbl;
     const int tpos = is_v ? t : (PF_BN / 2) * (int)rank + t;   // position within the tile
     // V tile buffers [D/128][64 rows][128 B]; K pair buffers [D/64][64 rows][128 B]
     uint8_t* dst_base = (is_v ? sV : sK) + kbl * (PF_BN * 128) + t * 128;
-    const int64_t code_off = (is_v ? a.codes_region : 0) + kb * 32 + u0 * 16;
-    // affine: the block's scale/bias word; TQ4: the vector's fp16 norm
-    const int64_t sb_off = a.sb_base + (is_v ? a.sb_region : 0) + (TQ ? 0 : kb * 4);
     const uint32_t lut_lane = smem_u32(sm + L::OFF_LUT) + 4u * (uint32_t)lane;
-    struct Tile {
-      uint4 c[UPI];
-      uint32_t sbw;
-      bool valid;
-    };
-    // page id of tile j (P >= 64, so a tile lies in one page); it is loaded a
-    // step before its tile's code loads need it
-    // j: local tile index; the history tile is jb + j
-    auto page_of = [&](int j) -> int {
-      return j < ntiles ? __ldg(pt + ((jb + j) * PF_BN) / a.P) : -1;
-    };
-    auto load_tile = [&](int j, int page, Tile& x) {
-      const int key0 = (jb + j) * PF_BN;
-      const bool pok = page >= 0 && page < a.num_pages;
-      if (!pok && dt == 0) flag_error(a.status, JF_DEV_ERR_PAGE_ID);
-      x.valid = pok && (key0 + tpos < kmax_pair);
-      if (x.valid) {
-        const uint8_t* base = a.pool + (int64_t)page * a.page_bytes;
-        const int64_t row = (int64_t)kvh * a.P + key0 % a.P + tpos;
-        const uint8_t* cp = base + code_off + row * CB;
+    const uint8_t* const stg = sm + L::OFF_STG + (is_v ? L::BOX_BYTES : 0);
+    // affine: the block's scale/bias word; TQ4: the vector's fp16 norm
+    const uint8_t* const side = sm + L::OFF_SIDE + ((is_v ? PF_BN / 2 : 0) + t) * L::SBB +
+                                (TQ ? 0 : kb * 4);
+    // this thread's 16-byte chunks of a stage: rows are swizzled over their
+    // length (128, 64 or 32 bytes)
+    uint32_t scol[UPI];
 #pragma unroll
-        for (int u = 0; u < UPI; ++u) x.c[u] = __ldg(reinterpret_cast<const uint4*>(cp + 16 * u));
-        if constexpr (TQ)
-          x.sbw = __ldg(reinterpret_cast<const uint16_t*>(base + sb_off + row * 2));
-        else
-          x.sbw = __ldg(reinterpret_cast<const uint32_t*>(base + sb_off + row * SBB));
-      }
-    };
-    auto store = [&](uint8_t* tile, const Tile& x) {
+    for (int u = 0; u < UPI; ++u) {
+      const int ch = unit * UPI + u, row = t;
+      const int len = is_v ? CB / 2 : CB;
+      const int x = len == 128 ? row & 7 : len == 64 ? (row >> 1) & 3 : (row >> 2) & 1;
+      scol[u] = (uint32_t)(row * len + ((ch ^ x) << 4));
+    }
+    auto store = [&](uint8_t* tile, const uint4 (&c)[UPI], uint32_t sbw, bool valid) {
       uint4 o[UPI][4];
       if constexpr (TQ) {
         // TQ4: norm * centroid of each index, natural d order (byte i gives
         // d 2i, 2i+1); |c| < 1/4 and norm <= 65504 keep it in fp16 range
-        const uint32_t n2 = (x.sbw & 0xFFFFu) | (x.sbw << 16);
+        const uint32_t n2 = valid ? sbw | (sbw << 16) : 0u;
 #pragma unroll
         for (int u = 0; u < UPI; ++u) {
-          const uint32_t cw[4] = {x.c[u].x, x.c[u].y, x.c[u].z, x.c[u].w};
+          const uint32_t cw[4] = {c[u].x, c[u].y, c[u].z, c[u].w};
 #pragma unroll
           for (int w = 0; w < 4; ++w) {
             uint32_t q4[4];
@@ -468,14 +492,14 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
         }
       } else {
         uint32_t s2, b2;
-        sb_to_h2(x.sbw, s2, b2);
+        sb_to_h2(valid ? sbw : 0u, s2, b2);   // 0 * code + 0 past the history
         // K and V are rebuilt in fp16: a group whose values can leave its
         // range (|bias| + 15 scale >= 65504, or a non-finite word) is reported
-        if (x.valid && !(fabsf(bf16hi_to_f32(x.sbw)) + 15.f * bf16lo_to_f32(x.sbw) < 65504.f))
+        if (valid && !(fabsf(bf16hi_to_f32(sbw)) + 15.f * bf16lo_to_f32(sbw) < 65504.f))
           flag_error(a.status, JF_DEV_ERR_RANGE);
 #pragma unroll
         for (int u = 0; u < UPI; ++u) {
-          const uint32_t cw[4] = {x.c[u].x, x.c[u].y, x.c[u].z, x.c[u].w};
+          const uint32_t cw[4] = {c[u].x, c[u].y, c[u].z, c[u].w};
 #pragma unroll
           for (int w = 0; w < 4; ++w) o[u][w] = dequant8(cw[w], s2, b2);
         }
@@ -485,28 +509,36 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
           const int cc = (u0 + u) * 4 + w;
-          *reinterpret_cast<uint4*>(tile + ((cc ^ (t & 7)) << 4)) =
-              x.valid ? o[u][w] : make_uint4(0, 0, 0, 0);
+          *reinterpret_cast<uint4*>(tile + ((cc ^ (t & 7)) << 4)) = o[u][w];
         }
     };
-    // Three register tiles rotate by name (the loop is unrolled by 3), so the
-    // loads for tile j + 2 stay in flight while tile j is converted.
-    Tile ta, tb, tcur;
     bool ok = true;
-    int pg_next = page_of(2);
     // K warps: tile j's half goes to rows 32 (j & 1) .. of pair buffer
     // (j / 2) % 2, free once S of the pair two back is done; V warps: tile
-    // buffer j % VB, free once P V of tile j - VB is done.  The
-    // loads of tile j + 2 are issued after tile j's arrive: a release waits
-    // for every earlier access of the warp, so loads still in flight would
-    // hold the arrive back by a memory latency.
+    // buffer j % VB, free once P V of tile j - VB is done.  These warps touch
+    // no global memory: a release waits for every earlier access of the warp,
+    // so a load in flight would hold the arrive back by a memory latency.
     // (one call of store per step: the roles share the SM's instruction cache)
-    auto step = [&](int j, const Tile& cur, Tile& nxt) {
+    int sst = 0;               // stage of tile j
+    uint32_t spar = 0;         // and its parity
+    for (int j = 0; j < ntiles; ++j) {
       const int kbuf = j % L::VB, pb = (j >> 1) & 1;
+      if (!mbar_wait_bounded(&stg_full[sst], spar)) { ok = false; break; }
+      uint4 c[UPI];
+#pragma unroll
+      for (int u = 0; u < UPI; ++u)
+        c[u] = *reinterpret_cast<const uint4*>(stg + sst * (2 * L::BOX_BYTES) + scol[u]);
+      const uint32_t sbw = TQ ? *reinterpret_cast<const uint16_t*>(side + sst * L::SIDE_BYTES)
+                              : *reinterpret_cast<const uint32_t*>(side + sst * L::SIDE_BYTES);
+      const bool valid = stg_ok[sst] != 0 && (jb + j) * PF_BN + tpos < kmax_pair;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&stg_free[sst]);
+      if (++sst == L::NST) { sst = 0; spar ^= 1u; }
       uint64_t* const free_bar = is_v ? &pv_done[(j - L::VB) & 3] : &s_full[pb];
       const uint32_t free_par = is_v ? ((j - L::VB) >> 2) & 1 : (((j >> 1) - 2) >> 1) & 1;
-      if (j >= (is_v ? L::VB : 4) && !tc::wait_cluster(free_bar, free_par)) { ok = false; return; }
-      store(dst_base + (is_v ? kbuf * L::VT_BYTES : pb * L::KP_BYTES + (j & 1) * (32 * 128)), cur);
+      if (j >= (is_v ? L::VB : 4) && !tc::wait_cluster(free_bar, free_par)) { ok = false; break; }
+      store(dst_base + (is_v ? kbuf * L::VT_BYTES : pb * L::KP_BYTES + (j & 1) * (32 * 128)), c,
+            sbw, valid);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
@@ -515,17 +547,47 @@ prefill_kernel(const __grid_constant__ PrefillArgs a) {
         // a last K half without a partner tile arrives for it too
         if (!is_v && (j & 1) == 0 && j + 1 == ntiles) tc::arrive_cluster(full_bar, 0);
       }
-      if (j + 2 < ntiles) load_tile(j + 2, pg_next, nxt);
-      pg_next = page_of(j + 3);
-    };
-    if (ntiles > 0) load_tile(0, page_of(0), ta);
-    if (ntiles > 1) load_tile(1, page_of(1), tb);
-    for (int j = 0; j < ntiles && ok; j += 3) {
-      step(j, ta, tcur);
-      if (j + 1 < ntiles && ok) step(j + 1, tb, ta);
-      if (j + 2 < ntiles && ok) step(j + 2, tcur, tb);
     }
     if (!ok && dt == 0) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
+  } else if (warp == PF_TMA_WARP) {
+    // ================= code copies (TMA producer) =================
+    if (lane == 0) {
+      bool ok = true;
+      int j = 0;
+      int page = ntiles > 0 ? __ldg(pt + ((jb * PF_BN) >> a.log2P)) : -1;
+      for (; j < ntiles; ++j) {
+        const int st = j % L::NST;
+        const int key0 = (jb + j) * PF_BN;
+        const int next = j + 1 < ntiles ? __ldg(pt + ((key0 + PF_BN) >> a.log2P)) : -1;
+        if (j >= L::NST && !mbar_wait_bounded(&stg_free[st], (j / L::NST - 1) & 1)) { ok = false; break; }
+        uint64_t* const bar = &stg_full[st];
+        uint8_t* const dst = sm + L::OFF_STG + st * (2 * L::BOX_BYTES);
+        uint8_t* const sdst = sm + L::OFF_SIDE + st * L::SIDE_BYTES;
+        const bool pok = page >= 0 && page < a.num_pages;
+        stg_ok[st] = pok ? 1 : 0;
+        if (pok) {
+          const int slot = key0 & (a.P - 1);
+          const int kslot = slot + (PF_BN / 2) * (int)rank;   // this CTA's K half
+          const uint8_t* const gside = a.pool + (int64_t)page * a.page_bytes + a.sb_base;
+          const int64_t row0 = (int64_t)kvh * a.P;
+          mbar_arrive_expect_tx(bar, L::STAGE_TX);
+          tma_load_5d(dst, &kmap, 0, kslot, kvh, 0, page, bar);
+          tma_load_5d(dst + L::BOX_BYTES, &vmap, (CB / 2) * (int)rank, slot, kvh, 1, page, bar);
+          bulk_g2s(sdst, gside + (row0 + kslot) * L::SBB, PF_BN / 2 * L::SBB, bar);
+          bulk_g2s(sdst + PF_BN / 2 * L::SBB, gside + a.sb_region + (row0 + slot) * L::SBB,
+                   PF_BN * L::SBB, bar);
+        } else {
+          flag_error(a.status, JF_DEV_ERR_PAGE_ID);
+          mbar_arrive(bar);
+        }
+        page = next;
+      }
+      if (!ok) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
+      // copies still in flight land before the CTA can exit
+      for (int i = j > L::NST ? j - L::NST : 0; i < j; ++i)
+        mbar_wait_bounded(&stg_full[i % L::NST], (i / L::NST) & 1, 1u << 16);
+    }
+    __syncwarp();
   } else {
     // ================= softmax + epilogue (this CTA's 128 rows) =================
     // Rows past the chunk (padding) see every position: their Q rows are zero
@@ -800,17 +862,20 @@ size_t prefill_workspace_bytes(int64_t rows, int64_t Hq, int64_t D, int64_t S, i
 // One prefill launch of a given instantiation (its shared-memory opt-in is
 // set once per instantiation and device).
 template <int D, int FMT>
-static int launch_pf(const dim3& grid, const PrefillArgs& a, cudaStream_t stream) {
+static int launch_pf(const dim3& grid, const CUtensorMap* maps, const PrefillArgs& a,
+                     cudaStream_t stream) {
   if (smem_optin((const void*)prefill_kernel<D, FMT>, PfSmem<D, FMT>::TOTAL) != JF_OK)
     return JF_ERR_CUDA;
-  prefill_kernel<D, FMT><<<grid, PF_THREADS, PfSmem<D, FMT>::TOTAL, stream>>>(a);
+  prefill_kernel<D, FMT><<<grid, PF_THREADS, PfSmem<D, FMT>::TOTAL, stream>>>(maps[0], maps[1],
+                                                                          a);
   return cudaGetLastError() == cudaSuccess ? JF_OK : JF_ERR_CUDA;
 }
 
 // One launch over the chunks of `nreq` requests (nreq <= PF_MAX_REQ); requests
 // with an empty chunk get no CTAs.  The request with the most attended
 // positions goes first, so the longest CTA pairs start earliest.
-int launch_prefill_batch(const Geom& g, const jf_kv_pool& pool, const int32_t* const* pt_rows,
+int launch_prefill_batch(const Geom& g, const jf_kv_pool& pool, const CUtensorMap* maps,
+                         const int32_t* const* pt_rows,
                          const int32_t* q_start, const int32_t* chunk_len, const void* q,
                          const int64_t* q_row0, int32_t nreq, int32_t Hq, float softmax_scale,
                          int32_t causal, void* out, void* workspace, cudaStream_t stream,
@@ -826,6 +891,7 @@ int launch_prefill_batch(const Geom& g, const jf_kv_pool& pool, const int32_t* c
   a.sb_base = 2 * g.codes_region;
   a.sb_region = g.sb_region;
   a.P = g.P;
+  a.log2P = __builtin_ctz((unsigned)g.P);
   a.Hkv = g.Hkv;
   a.Hq = Hq;
   a.G = Hq / g.Hkv;
@@ -895,11 +961,11 @@ int launch_prefill_batch(const Geom& g, const jf_kv_pool& pool, const int32_t* c
   }
   int st;
   if (g.D == 256)
-    st = tq ? launch_pf<256, JF_FMT_TQ4>(grid, a, stream)
-            : launch_pf<256, JF_FMT_AFFINE4_G64>(grid, a, stream);
+    st = tq ? launch_pf<256, JF_FMT_TQ4>(grid, maps, a, stream)
+            : launch_pf<256, JF_FMT_AFFINE4_G64>(grid, maps, a, stream);
   else
-    st = tq ? launch_pf<128, JF_FMT_TQ4>(grid, a, stream)
-            : launch_pf<128, JF_FMT_AFFINE4_G64>(grid, a, stream);
+    st = tq ? launch_pf<128, JF_FMT_TQ4>(grid, maps, a, stream)
+            : launch_pf<128, JF_FMT_AFFINE4_G64>(grid, maps, a, stream);
   if (st) return st;
   if (num_splits > 1 || tq) {
     uint16_t* o = static_cast<uint16_t*>(out);
@@ -923,14 +989,8 @@ int launch_prefill_batch(const Geom& g, const jf_kv_pool& pool, const int32_t* c
   return JF_OK;
 }
 
-int launch_prefill(const Geom& g, const jf_kv_pool& pool, const CUtensorMap&,
-                   const int32_t* page_table_row, const void* q, int32_t q_start,
-                   int32_t chunk_len, int32_t Hq, float softmax_scale, int32_t causal, void* out,
-                   void* workspace, cudaStream_t stream) {
-  const int64_t row0 = 0;
-  return launch_prefill_batch(g, pool, &page_table_row, &q_start, &chunk_len, q, &row0, 1, Hq,
-                              softmax_scale, causal, out, workspace, stream, 1, chunk_len,
-                              nullptr);
-}
+// rows of the code boxes that the dequantization warps copy: K (whole rows of
+// D/2 bytes) and V (half rows)
+int prefill_box_rows(bool v) { return v ? PF_BN : PF_BN / 2; }
 
 }  // namespace jfkv
