@@ -33,22 +33,23 @@
 //               [D, D + 256); P_j (fp16) overwrites S columns already read.
 //               S over two tiles keeps the MMA at N = 128 (an N = 64 pair
 //               MMA takes as long as an N = 128 one).
-//   warps 1-8   dequantize this CTA's halves of 64-position K/V tiles
+//   dequantize  (8 warps, TQ4 16) this CTA's halves of 64-position K/V tiles
 //               (4-bit codes -> fp16 integers through the mantissa of fp16
 //               1024, then x = code * scale + bias with one fused
 //               multiply-add) into 128B-swizzled buffers, one item (one
-//               position's code bytes of a 64-wide block) per thread; warps
-//               1-4 write K halves into two pair buffers (free again once S of
-//               the pair two back is done), warps 5-8 V halves into four
-//               tile buffers (free once P V of the tile four back is done),
-//               each arriving on CTA 0's K-pair or V-tile barrier.
-//   warps 9-12  one thread per row: Q row -> shared memory at the start;
+//               position's code bytes of a 64-wide block) per thread; the
+//               first four warps of 8 write K halves into two pair buffers
+//               (free again once S of the pair two back is done), the others
+//               V halves into four tile buffers (free once P V of the tile
+//               four back is done), each arriving on CTA 0's K-pair or V-tile
+//               barrier.
+//   softmax     (4 warps) one thread per row: Q row -> shared memory at the start;
 //               online softmax on S (tcgen05.ld), P back to TMEM as fp16
 //               over S columns already read (tcgen05.st) and an arrive on
 //               CTA 0's P barrier; the running maximum is moved only when it
 //               grows by more than 2^8, and then O is rescaled in TMEM;
 //               finally O / l -> bf16 output.
-//   warp 13     one lane copies the packed codes and side words of the tiles
+//   warp 1      one lane copies the packed codes and side words of the tiles
 //               ahead from the pool into a ring of NST stages by TMA (it also
 //               looks the pages up).  The dequantization warps, the slowest
 //               link of the chain, then touch no global memory and no
@@ -61,7 +62,13 @@
 //               us with the copies issued by each of those warps, 1,528 us from
 //               here).  With the two changes above that case went from 1,525
 //               to 1,196 us, 8 chunks of 64 queries after 4K-32K positions from
-//               354 to 269 us.
+//               354 to 269 us; with fewer instructions around each wait (mapped
+//               addresses, several polls a loop step, three-input maxima) to
+//               1,190 and 264 us.  What bounds it now: shared memory (the
+//               operands of S and P V, the rebuilt tiles' stores and the codes
+//               take ~2,030 of the ~3,200 cycles a tile pair and CTA takes) and
+//               issue slots (dequantization and softmax, 56 %); the tensor work
+//               alone is ~2,040 cycles.
 // Within every 8 consecutive d the tiles store elements in the order
 // 0,4,1,5,2,6,3,7 (the pairs one 32-bit word of codes yields); Q uses the same
 // order, so Q K^T is unchanged, and the epilogue undoes it for O.  Q is
@@ -76,10 +83,8 @@ namespace jfkv {
 
 constexpr int PF_BM = 128;   // MMA rows per CTA (256 per CTA pair)
 constexpr int PF_BN = 64;    // positions per K/V tile
-constexpr int PF_DQ_WARPS = 8;
+constexpr int PF_DQ_WARPS = 8;    // per set
 constexpr int PF_SM_WARPS = 4;   // one per TMEM lane quarter, one row per thread
-constexpr int PF_THREADS = 32 * (2 + PF_DQ_WARPS + PF_SM_WARPS);
-constexpr int PF_TMA_WARP = 1 + PF_DQ_WARPS + PF_SM_WARPS;   // the code copies' producer
 constexpr int PF_KVBUF = 4;     // P V completion barriers, by tile index mod 4
 constexpr float PF_TAU = 8.f;   // log2 headroom before the running max moves
 
@@ -144,6 +149,29 @@ struct PfSmem {
   static constexpr int OFF_LUT = OFF_BAR + 256;   // TQ4 centroid table (lane-replicated)
   static constexpr int TOTAL = 1024 + OFF_LUT + (TQ ? 256 * 32 * 4 : 0);
   static_assert(TOTAL <= 227 * 1024, "shared memory per CTA");
+};
+
+// Warps: 0 MMA, 1 code copies, 2-3 idle, then dequantization and softmax, each
+// whole warpgroups.  TQ4 runs two sets of dequantization warps, one for the
+// even and one for the odd tiles: its centroid lookups wait on shared memory
+// (1,500 queries after 20,001 positions: 641 us with one set, 604 with two).
+// The affine conversion is bound by issue slots, and a second set only takes
+// them from the softmax (2,048 after 30,720: 1,189 against 1,257 us).
+// Two sets need a register split: every thread starts with LAUNCH_REGS, and
+// the softmax warpgroup's increase comes out of the others' decrease.
+template <int FMT>
+struct PfRoles {
+  static constexpr int SETS = FMT == JF_FMT_TQ4 ? 2 : 1;
+  static constexpr int TMA_WARP = 1;
+  static constexpr int DQ0 = 4;
+  static constexpr int SM0 = DQ0 + SETS * PF_DQ_WARPS;
+  static constexpr int THREADS = 32 * (SM0 + PF_SM_WARPS);
+  static constexpr bool SPLIT_REGS = SETS > 1;
+  static constexpr int LAUNCH_REGS = 80, MMA_REGS = 48, DQ_REGS = 72, SM_REGS = 136;
+  static_assert(!SPLIT_REGS || 32 * (DQ0 * MMA_REGS + SETS * PF_DQ_WARPS * DQ_REGS +
+                                     PF_SM_WARPS * SM_REGS) <= THREADS * LAUNCH_REGS,
+                "register shares exceed the launch's");
+  static_assert(SM0 % 4 == 0, "a softmax warp's id gives its TMEM lane quarter");
 };
 
 // packed fp32 pairs (Blackwell f32x2 arithmetic)
@@ -213,10 +241,11 @@ __device__ __forceinline__ void sb_to_h2(uint32_t w, uint32_t& s2, uint32_t& b2)
 // FMT: JF_FMT_AFFINE4_G64, or JF_FMT_TQ4 (centroid table, rotated queries,
 // natural d order, partial outputs rotated back by the merge kernel)
 template <int D, int FMT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PfRoles<FMT>::THREADS, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                const __grid_constant__ PrefillArgs a) {
   using L = PfSmem<D, FMT>;
+  using R = PfRoles<FMT>;
   constexpr bool TQ = FMT == JF_FMT_TQ4;
   constexpr int NKB = D / 64;           // 64-wide d blocks
   constexpr int UPI = (D == 256) ? 2 : 1;   // 16-byte code units per dequant item
@@ -247,7 +276,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   uint64_t* stg_full = bars + 18;                // [NST] a tile's code bytes have landed
   uint64_t* stg_free = bars + 18 + L::NST;       // [NST] ... and have been read
-  int32_t* stg_ok = reinterpret_cast<int32_t*>(bars + 18 + 2 * L::NST);   // [NST] page id was valid
+  int32_t* stg_n = reinterpret_cast<int32_t*>(bars + 18 + 2 * L::NST);   // [NST] positions of the tile that hold data
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_rank();
@@ -332,7 +361,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     return reinterpret_cast<uint4*>(sQ + (m >> 3) * (PF_BM * 128) + r * 128 +
                                     (((m & 7) ^ (r & 7)) << 4));
   };
-  if (TQ && warp > PF_DQ_WARPS && warp < PF_TMA_WARP) {
+  if (TQ && warp >= R::SM0) {
     // rotated fp32 query row, natural d order (the centroid pairs are too)
     const float* qrow = a.qrot + ((int64_t)(rq.row0 + q0 + qi) * a.Hq + kvh * a.G + r % a.G) * D;
     float qmax = 0.f;
@@ -356,7 +385,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
                                pack_f16x2(w1.x * qs, w1.y * qs), pack_f16x2(w1.z * qs, w1.w * qs));
     }
     fence_proxy_async_smem();
-  } else if (warp > PF_DQ_WARPS && warp < PF_TMA_WARP) {
+  } else if (warp >= R::SM0) {
     const uint16_t* qrow = rq.q + ((int64_t)(q0 + qi) * a.Hq + kvh * a.G + r % a.G) * D;
     float qmax = 0.f;
     if (row_ok) {
@@ -389,6 +418,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
   tc::cluster_sync();   // both CTAs' Q rows are in shared memory before the first MMA
   tc::fence_after();
 
+  if (warp < R::DQ0) {
+  if constexpr (R::SPLIT_REGS) tc::setmaxnreg_dec<R::MMA_REGS>();
   if (warp == 0) {
     // ================= MMA issuer (CTA 0 of the pair) =================
     if (rank == 0) {
@@ -437,14 +468,56 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
       if (!ok && lane == 0) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
     }
     __syncwarp();
-  } else if (warp <= PF_DQ_WARPS) {
+  } else if (warp == R::TMA_WARP) {
+    // ================= code copies (TMA producer) =================
+    if (lane == 0) {
+      bool ok = true;
+      int j = 0;
+      int page = ntiles > 0 ? __ldg(pt + ((jb * PF_BN) >> a.log2P)) : -1;
+      for (; j < ntiles; ++j) {
+        const int st = j % L::NST;
+        const int key0 = (jb + j) * PF_BN;
+        const int next = j + 1 < ntiles ? __ldg(pt + ((key0 + PF_BN) >> a.log2P)) : -1;
+        if (j >= L::NST && !tc::wait_cta_idle_at(smem_u32(&stg_free[st]), (j / L::NST - 1) & 1)) { ok = false; break; }
+        uint64_t* const bar = &stg_full[st];
+        uint8_t* const dst = sm + L::OFF_STG + st * (2 * L::BOX_BYTES);
+        uint8_t* const sdst = sm + L::OFF_SIDE + st * L::SIDE_BYTES;
+        const bool pok = page >= 0 && page < a.num_pages;
+        stg_n[st] = pok ? kmax_pair - key0 : 0;
+        if (pok) {
+          const int slot = key0 & (a.P - 1);
+          const int kslot = slot + (PF_BN / 2) * (int)rank;   // this CTA's K half
+          const uint8_t* const gside = a.pool + (int64_t)page * a.page_bytes + a.sb_base;
+          const int64_t row0 = (int64_t)kvh * a.P;
+          mbar_arrive_expect_tx(bar, L::STAGE_TX);
+          tma_load_5d(dst, &kmap, 0, kslot, kvh, 0, page, bar);
+          tma_load_5d(dst + L::BOX_BYTES, &vmap, (CB / 2) * (int)rank, slot, kvh, 1, page, bar);
+          bulk_g2s(sdst, gside + (row0 + kslot) * L::SBB, PF_BN / 2 * L::SBB, bar);
+          bulk_g2s(sdst + PF_BN / 2 * L::SBB, gside + a.sb_region + (row0 + slot) * L::SBB,
+                   PF_BN * L::SBB, bar);
+        } else {
+          flag_error(a.status, JF_DEV_ERR_PAGE_ID);
+          mbar_arrive(bar);
+        }
+        page = next;
+      }
+      if (!ok) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
+      // copies still in flight land before the CTA can exit
+      for (int i = j > L::NST ? j - L::NST : 0; i < j; ++i)
+        mbar_wait_bounded(&stg_full[i % L::NST], (i / L::NST) & 1, 1u << 16);
+    }
+    __syncwarp();
+  }
+  } else if (warp < R::SM0) {
+    if constexpr (R::SPLIT_REGS) tc::setmaxnreg_dec<R::DQ_REGS>();
     // ================= dequantization (this CTA's halves) =================
     // One item per thread: the code bytes of one position, 16 UPI of them.
     // K warp w: positions 32 rank + 8 w .. + 7 of the tile, whole rows (4 items
     // each); V warp w: positions 16 w .. + 15, this CTA's half rows (2 items).
-    const int dt = (int)threadIdx.x - 32;
+    const int set = (warp - R::DQ0) / PF_DQ_WARPS;   // takes the tiles j % SETS == set
+    const int dt = (int)threadIdx.x - 32 * (R::DQ0 + set * PF_DQ_WARPS);
     const bool is_v = dt >= 128;
-    const int dw = (warp - 1) & 3;
+    const int dw = (warp - R::DQ0) & 3;
     const int t = is_v ? 16 * dw + (lane & 15) : 8 * dw + (lane & 7);
     const int unit = is_v ? lane >> 4 : lane >> 3;
     const int kbl = (UPI == 2) ? unit : unit >> 1;
@@ -519,76 +592,42 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     // no global memory: a release waits for every earlier access of the warp,
     // so a load in flight would hold the arrive back by a memory latency.
     // (one call of store per step: the roles share the SM's instruction cache)
-    int sst = 0;               // stage of tile j
+    const uint32_t free0 = smem_u32(is_v ? pv_done : s_full);
+    const uint32_t full0 = tc::map_rank0(smem_u32(is_v ? v_full : k_full));
+    uint8_t* const dst0 = dst_base;
+    int sst = set;             // stage of tile j
     uint32_t spar = 0;         // and its parity
-    for (int j = 0; j < ntiles; ++j) {
-      const int kbuf = j % L::VB, pb = (j >> 1) & 1;
-      if (!mbar_wait_bounded(&stg_full[sst], spar)) { ok = false; break; }
+    for (int j = set; j < ntiles; j += R::SETS) {
+      if (!tc::wait_cta_at(smem_u32(&stg_full[sst]), spar)) { ok = false; break; }
       uint4 c[UPI];
 #pragma unroll
       for (int u = 0; u < UPI; ++u)
         c[u] = *reinterpret_cast<const uint4*>(stg + sst * (2 * L::BOX_BYTES) + scol[u]);
       const uint32_t sbw = TQ ? *reinterpret_cast<const uint16_t*>(side + sst * L::SIDE_BYTES)
                               : *reinterpret_cast<const uint32_t*>(side + sst * L::SIDE_BYTES);
-      const bool valid = stg_ok[sst] != 0 && (jb + j) * PF_BN + tpos < kmax_pair;
+      const bool valid = tpos < stg_n[sst];
       __syncwarp();
       if (lane == 0) mbar_arrive(&stg_free[sst]);
-      if (++sst == L::NST) { sst = 0; spar ^= 1u; }
-      uint64_t* const free_bar = is_v ? &pv_done[(j - L::VB) & 3] : &s_full[pb];
-      const uint32_t free_par = is_v ? ((j - L::VB) >> 2) & 1 : (((j >> 1) - 2) >> 1) & 1;
-      if (j >= (is_v ? L::VB : 4) && !tc::wait_cluster(free_bar, free_par)) { ok = false; break; }
-      store(dst_base + (is_v ? kbuf * L::VT_BYTES : pb * L::KP_BYTES + (j & 1) * (32 * 128)), c,
-            sbw, valid);
+      if ((sst += R::SETS) >= L::NST) { sst -= L::NST; spar ^= 1u; }
+      const int pb = (j >> 1) & 1;
+      const int back = is_v ? j - L::VB : j - 4;   // a buffer's last use: the parity of j / 4 then
+      const uint32_t fb = free0 + 8 * (is_v ? back & 3 : pb);
+      if (back >= 0 && !tc::wait_cluster_at(fb, (back >> 2) & 1)) { ok = false; break; }
+      const int vb = j % L::VB;
+      store(dst0 + (is_v ? vb * L::VT_BYTES : pb * L::KP_BYTES + (j & 1) * (32 * 128)), c, sbw,
+            valid);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
-        uint64_t* const full_bar = is_v ? &v_full[kbuf] : &k_full[pb];
-        tc::arrive_cluster(full_bar, 0);
+        const uint32_t fl = full0 + 8 * (is_v ? vb : pb);
+        tc::arrive_mapped(fl);
         // a last K half without a partner tile arrives for it too
-        if (!is_v && (j & 1) == 0 && j + 1 == ntiles) tc::arrive_cluster(full_bar, 0);
+        if (!is_v && (j & 1) == 0 && j + 1 == ntiles) tc::arrive_mapped(fl);
       }
     }
     if (!ok && dt == 0) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
-  } else if (warp == PF_TMA_WARP) {
-    // ================= code copies (TMA producer) =================
-    if (lane == 0) {
-      bool ok = true;
-      int j = 0;
-      int page = ntiles > 0 ? __ldg(pt + ((jb * PF_BN) >> a.log2P)) : -1;
-      for (; j < ntiles; ++j) {
-        const int st = j % L::NST;
-        const int key0 = (jb + j) * PF_BN;
-        const int next = j + 1 < ntiles ? __ldg(pt + ((key0 + PF_BN) >> a.log2P)) : -1;
-        if (j >= L::NST && !mbar_wait_bounded(&stg_free[st], (j / L::NST - 1) & 1)) { ok = false; break; }
-        uint64_t* const bar = &stg_full[st];
-        uint8_t* const dst = sm + L::OFF_STG + st * (2 * L::BOX_BYTES);
-        uint8_t* const sdst = sm + L::OFF_SIDE + st * L::SIDE_BYTES;
-        const bool pok = page >= 0 && page < a.num_pages;
-        stg_ok[st] = pok ? 1 : 0;
-        if (pok) {
-          const int slot = key0 & (a.P - 1);
-          const int kslot = slot + (PF_BN / 2) * (int)rank;   // this CTA's K half
-          const uint8_t* const gside = a.pool + (int64_t)page * a.page_bytes + a.sb_base;
-          const int64_t row0 = (int64_t)kvh * a.P;
-          mbar_arrive_expect_tx(bar, L::STAGE_TX);
-          tma_load_5d(dst, &kmap, 0, kslot, kvh, 0, page, bar);
-          tma_load_5d(dst + L::BOX_BYTES, &vmap, (CB / 2) * (int)rank, slot, kvh, 1, page, bar);
-          bulk_g2s(sdst, gside + (row0 + kslot) * L::SBB, PF_BN / 2 * L::SBB, bar);
-          bulk_g2s(sdst + PF_BN / 2 * L::SBB, gside + a.sb_region + (row0 + slot) * L::SBB,
-                   PF_BN * L::SBB, bar);
-        } else {
-          flag_error(a.status, JF_DEV_ERR_PAGE_ID);
-          mbar_arrive(bar);
-        }
-        page = next;
-      }
-      if (!ok) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
-      // copies still in flight land before the CTA can exit
-      for (int i = j > L::NST ? j - L::NST : 0; i < j; ++i)
-        mbar_wait_bounded(&stg_full[i % L::NST], (i / L::NST) & 1, 1u << 16);
-    }
-    __syncwarp();
   } else {
+    if constexpr (R::SPLIT_REGS) tc::setmaxnreg_inc<R::SM_REGS>();
     // ================= softmax + epilogue (this CTA's 128 rows) =================
     // Rows past the chunk (padding) see every position: their Q rows are zero
     // and their outputs are never stored, and keeping them unmasked keeps the
@@ -602,7 +641,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
       // columns 64 + 32 (j & 1) .. of its pair's S/P buffer; P_j (fp16)
       // goes to columns 32 (j & 1) .. once both are read
       const int pi = j >> 1;
-      if (!tc::wait_cluster(&s_full[pi & 1], (pi >> 1) & 1)) { ok = false; break; }
+      if ((j & 1) == 0 && !tc::wait_cluster(&s_full[pi & 1], (pi >> 1) & 1)) { ok = false; break; }
       tc::fence_after();
       const uint32_t tb = tS + (pi & 1) * (2 * PF_BN);
       uint32_t s0[32], s1[32];
@@ -629,7 +668,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
           for (int c = 0; c < PF_BN; ++c) x[c] *= smul;
         }
 #pragma unroll
-        for (int c = 0; c < PF_BN; ++c) m4[c & 3] = fmaxf(m4[c & 3], x[c]);
+        for (int c = 0; c < PF_BN; c += 2) m4[(c >> 1) & 3] = tc::max3(m4[(c >> 1) & 3], x[c], x[c + 1]);
         mt = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
       }
       const bool need = mt > m_ref + PF_TAU;
@@ -866,7 +905,15 @@ static int launch_pf(const dim3& grid, const CUtensorMap* maps, const PrefillArg
                      cudaStream_t stream) {
   if (smem_optin((const void*)prefill_kernel<D, FMT>, PfSmem<D, FMT>::TOTAL) != JF_OK)
     return JF_ERR_CUDA;
-  prefill_kernel<D, FMT><<<grid, PF_THREADS, PfSmem<D, FMT>::TOTAL, stream>>>(maps[0], maps[1],
+  if (PfRoles<FMT>::SPLIT_REGS) {   // a split of more than the launch has would wait forever
+    static const bool fits = [] {
+      cudaFuncAttributes fa;
+      return cudaFuncGetAttributes(&fa, (const void*)prefill_kernel<D, FMT>) == cudaSuccess &&
+             fa.numRegs >= PfRoles<FMT>::LAUNCH_REGS;
+    }();
+    if (!fits) return JF_ERR_CUDA;
+  }
+  prefill_kernel<D, FMT><<<grid, PfRoles<FMT>::THREADS, PfSmem<D, FMT>::TOTAL, stream>>>(maps[0], maps[1],
                                                                           a);
   return cudaGetLastError() == cudaSuccess ? JF_OK : JF_ERR_CUDA;
 }

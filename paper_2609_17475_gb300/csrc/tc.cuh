@@ -8,6 +8,7 @@
 namespace jfkv {
 namespace tc {
 
+
 // Shared-memory matrix descriptor, 128-byte swizzle (layout type 2), version 1.
 // addr/lbo/sbo in bytes (16-byte granularity).
 __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr, uint32_t lbo, uint32_t sbo) {
@@ -25,6 +26,16 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr, uint32_t lbo, uin
 __host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N, int a_mn, int b_mn) {
   return (1u << 4) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// Registers per thread of the executing warpgroup (every warp of it calls this).
+template <int N>
+__device__ __forceinline__ void setmaxnreg_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void setmaxnreg_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(N));
 }
 
 __device__ __forceinline__ void fence_before() {
@@ -114,19 +125,66 @@ __device__ __forceinline__ void arrive_cluster(uint64_t* bar, uint32_t rank) {
                ::"r"(remote) : "memory");
 }
 
+// The same with the address already mapped to CTA 0 (map_rank0), for loops
+// whose barriers are an offset from one base.
+__device__ __forceinline__ uint32_t map_rank0(uint32_t addr) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(remote) : "r"(addr));
+  return remote;
+}
+__device__ __forceinline__ void arrive_mapped(uint32_t remote) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];\n"
+               ::"r"(remote) : "memory");
+}
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // Bounded wait with cluster-scope acquire (for barriers other CTAs arrive on).
+// Four polls to a step of the loop: the polls of waiting warps compete for
+// issue slots with the warps they wait for.
+#define JF_POLL(scope, hint)                                                                        \
+  asm volatile(                                                                               \
+      "{\n\t.reg .pred p;\n\t.reg .u32 c;\n\tmov.u32 c, %3;\n"                                 \
+      "POLL:\n\t"                                                                             \
+      "mbarrier.try_wait.parity.acquire." scope ".shared::cta.b64 p, [%1], %2" hint ";\n\t" \
+      "@p bra DONE;\n\t"                                                                      \
+      "mbarrier.try_wait.parity.acquire." scope ".shared::cta.b64 p, [%1], %2" hint ";\n\t" \
+      "@p bra DONE;\n\t"                                                                      \
+      "mbarrier.try_wait.parity.acquire." scope ".shared::cta.b64 p, [%1], %2" hint ";\n\t" \
+      "@p bra DONE;\n\t"                                                                      \
+      "mbarrier.try_wait.parity.acquire." scope ".shared::cta.b64 p, [%1], %2" hint ";\n\t" \
+      "@p bra DONE;\n\t"                                                                      \
+      "add.s32 c, c, -1;\n\tsetp.ne.s32 p, c, 0;\n\t@p bra POLL;\n"                           \
+      "DONE:\n\tmov.u32 %0, c;\n\t}\n"                                                       \
+      : "=r"(left) : "r"(addr), "r"(parity), "r"(steps) : "memory")
+
+__device__ __forceinline__ bool wait_cluster_at(uint32_t addr, uint32_t parity,
+                                                uint32_t steps = (1u << 20)) {
+  uint32_t left;
+  JF_POLL("cluster", "");
+  return left != 0;
+}
+__device__ __forceinline__ bool wait_cta_at(uint32_t addr, uint32_t parity,
+                                            uint32_t steps = (1u << 20)) {
+  uint32_t left;
+  JF_POLL("cta", "");
+  return left != 0;
+}
+// For a producer that runs ahead: each poll may sleep for up to a microsecond.
+__device__ __forceinline__ bool wait_cta_idle_at(uint32_t addr, uint32_t parity,
+                                                 uint32_t steps = (1u << 18)) {
+  uint32_t left;
+  JF_POLL("cta", ", 1000");
+  return left != 0;
+}
+#undef JF_POLL
 __device__ __forceinline__ bool wait_cluster(uint64_t* bar, uint32_t parity,
-                                             uint32_t limit = (1u << 22)) {
-  for (uint32_t i = 0; i < limit; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    if (ok) return true;
-  }
-  return false;
+                                             uint32_t steps = (1u << 20)) {
+  return wait_cluster_at(smem_u32(bar), parity, steps);
 }
 
 #define JF_R8(i) "=r"(v[i]), "=r"(v[i + 1]), "=r"(v[i + 2]), "=r"(v[i + 3]), "=r"(v[i + 4]), \
