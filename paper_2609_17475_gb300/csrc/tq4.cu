@@ -25,6 +25,7 @@
 // are those of the affine decode.
 #include <cmath>
 #include <cfloat>
+#include <cstring>
 #include <vector>
 
 #include "decode.cuh"
@@ -108,11 +109,18 @@ int tq4_make_params(const jf_tq4_codec* codec, int d, Tq4Params* p) {
   for (int k = 0; k < 14; ++k)
     if (!((double)p->tq[k + 1] - (double)p->tq[k] > 0x1p-12)) p->exact_all = 1;
   for (int j = 0; j < 8; ++j) p->sk[j] = p->sv[j] = 0u;
-  for (int j = 0; j < d; ++j) {
-    const int a = codec->signs_k[j], b = codec->signs_v[j];
-    if ((a != 1 && a != -1) || (b != 1 && b != -1)) return JF_ERR_INVALID_ARG;
-    if (a < 0) p->sk[j >> 5] |= 1u << (j & 31);
-    if (b < 0) p->sv[j >> 5] |= 1u << (j & 31);
+  // eight signs at a time (bytes 0x01 and 0xFF): a host call builds these masks
+  // each time, and one by one they took ~0.5 us of it
+  for (int j = 0; j < d; j += 8) {
+    const int8_t* src[2] = {codec->signs_k + j, codec->signs_v + j};
+    uint32_t* dst[2] = {p->sk, p->sv};
+    for (int i = 0; i < 2; ++i) {
+      uint64_t w;
+      std::memcpy(&w, src[i], 8);
+      const uint64_t neg = (w >> 7) & 0x0101010101010101ull;
+      if ((w ^ (neg * 0xFEu)) != 0x0101010101010101ull) return JF_ERR_INVALID_ARG;
+      dst[i][j >> 5] |= (uint32_t)((neg * 0x0102040810204080ull) >> 56) << (j & 31);
+    }
   }
   return JF_OK;
 }
