@@ -37,6 +37,7 @@
 #include <cmath>
 #include <cfloat>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -1146,33 +1147,58 @@ decode_span_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArgs a)
 }
 
 
-// Merge for one or a few requests: one CTA per (32-wide slice of head_dim,
+// Merge for one or a few requests: one CTA per (64-wide slice of head_dim,
 // query row, request); its 8 warps take interleaved splits and reduce through
 // shared memory, so even one request's merge is spread over the whole GPU.
-// The kernel is a chain of dependent loads, so it issues them all at once:
-// the context length, every (m, l) row and this thread's partial outputs for
-// up to MERGE_SG_BATCH splits are loaded before any is used; rows past the
-// split plan are loaded (the workspace holds num_splits rows) and then
-// ignored.
+// The kernel is a chain of latencies (a few hundred KB read from L2), so it
+// issues its loads at once: the context length, every (m, l) row and this
+// thread's partial outputs for up to 8 NB splits are loaded before any is
+// used; rows past the split plan are loaded (the workspace holds num_splits
+// rows) and then ignored.
+//
+// Its CTAs are placed while the split kernel's leave, as many on an SM as fit,
+// and so crowded onto the first SMs to fall free: 24 heads x 8 slices of 32
+// sat on a quarter of the chip.  Now 24 x 4 slices of 64, and the launch asks
+// for as much (unused) shared memory as lets one of them on an SM, or two where
+// there are more than SMs.  Device time of a call: 256K positions 52.0 -> 50.5
+// us (TQ4 65.1 -> 64.2), fused step at 35,841 positions 15.7 -> 14.7 us, two
+// requests of 196,608 + 131,072 64.6 -> 63.2 us.  Slices of 32 with two on an SM
+// had given 50.8, 64.5, 15.0 and 64.8 us.
 constexpr int MERGE_THREADS = 256;
-constexpr int MERGE_DSLICE = 32;
-constexpr int MERGE_NSG = MERGE_THREADS / MERGE_DSLICE;   // split groups
-constexpr int MERGE_SG_BATCH = 16;                        // splits per thread per batch
-constexpr int MERGE_MLB = MERGE_SG_BATCH * MERGE_NSG / 32;   // (m, l) rows per lane per batch
+constexpr int MERGE_DSLICE = 64;                          // two columns per thread
+constexpr int MERGE_NSG = MERGE_THREADS / (MERGE_DSLICE / 2);   // split groups
 
-template <int D, bool SPAN>
+// Loads that stay where they are written: the compiler may otherwise move the
+// partial outputs' loads behind the maximum that decides whether they are used,
+// a second memory round trip.
+__device__ __forceinline__ float2 ld_here(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_here(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];\n" : "=f"(v) : "l"(p));
+  return v;
+}
+
+// NB: splits per thread in a batch, the smallest of 5, 10 and 16 that holds
+// the plan's splits (38 of them need 5; loads past the plan still cost their
+// issue).
+template <int D, bool SPAN, int NB>
 __global__ void __launch_bounds__(MERGE_THREADS) decode_merge_sg_kernel(const DecodeArgs a) {
   // SPAN: partial rows of the span plan.  A template parameter: the span
   // branch in the single-request instance, though never taken, had slowed
   // the 256K call by ~1.2 us.
-  __shared__ float red[MERGE_NSG][MERGE_DSLICE];
+  constexpr int MLB = (NB * MERGE_NSG + 31) / 32;   // (m, l) rows per lane per batch
+  __shared__ float2 red[MERGE_NSG][MERGE_DSLICE / 2];
   // the next kernel in the stream may be scheduled now; it waits for this
   // grid to complete before it reads anything
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   // the split kernel's partials must be complete and visible
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   const int d0 = blockIdx.x * MERGE_DSLICE, hq = blockIdx.y, b = blockIdx.z;
-  const int t = threadIdx.x, dd = t % MERGE_DSLICE, sg = t / MERGE_DSLICE;
+  const int t = threadIdx.x, dd = t % (MERGE_DSLICE / 2), sg = t / (MERGE_DSLICE / 2);
   const int lane = t & 31;
   // partials of split s: row row0 + s * rs.  Per-request plans put them at
   // ((b Hq + hq) num_splits + s) and are known only after the context is
@@ -1212,21 +1238,27 @@ __global__ void __launch_bounds__(MERGE_THREADS) decode_merge_sg_kernel(const De
     S = nsplit_bal;
   }
   const float2* ml = reinterpret_cast<const float2*>(a.part_ml) + row0;
-  const float* po = a.part_o + row0 * D + d0 + dd;
+  const float2* po = reinterpret_cast<const float2*>(a.part_o + row0 * D + d0) + dd;
 
   const int ctx_raw = a.ctx[b];
-  float2 mlv[MERGE_MLB];
-  float ov[MERGE_SG_BATCH], mv[MERGE_SG_BATCH];
+  float2 mlv[MLB];
+  float2 ov[NB];
+  float mv[NB];
 #pragma unroll
-  for (int k = 0; k < MERGE_MLB; ++k) {
+  for (int k = 0; k < MLB; ++k) {
     const int s = lane + 32 * k;
-    mlv[k] = (s < S) ? ml[s * rs] : make_float2(-INFINITY, 0.f);
+    mlv[k] = make_float2(-INFINITY, 0.f);
+    if (s < S) mlv[k] = ld_here(ml + s * rs);
   }
 #pragma unroll
-  for (int u = 0; u < MERGE_SG_BATCH; ++u) {
+  for (int u = 0; u < NB; ++u) {
     const int s = sg + MERGE_NSG * u;
-    ov[u] = (s < S) ? po[s * rs * D] : 0.f;
-    mv[u] = (s < S) ? ml[s * rs].x : -INFINITY;
+    ov[u] = make_float2(0.f, 0.f);
+    mv[u] = -INFINITY;
+    if (s < S) {
+      ov[u] = ld_here(po + s * rs * (D / 2));
+      mv[u] = ld_here(&ml[s * rs].x);
+    }
   }
   int ctx = ctx_raw;
   const int64_t cap = (int64_t)a.pt_stride * a.P;
@@ -1246,48 +1278,63 @@ __global__ void __launch_bounds__(MERGE_THREADS) decode_merge_sg_kernel(const De
   // global maximum (every warp finds it itself)
   float M = -INFINITY;
 #pragma unroll
-  for (int k = 0; k < MERGE_MLB; ++k)
+  for (int k = 0; k < MLB; ++k)
     if (lane + 32 * k < nsplit) M = fmaxf(M, mlv[k].x);
-  for (int s = lane + 32 * MERGE_MLB; s < nsplit; s += 32) M = fmaxf(M, ml[s * rs].x);
+  for (int s = lane + 32 * MLB; s < nsplit; s += 32) M = fmaxf(M, ml[s * rs].x);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
 
-  float L = 0.f, acc = 0.f;
+  float L = 0.f;
+  float2 acc = make_float2(0.f, 0.f);
   if (M != -INFINITY) {
 #pragma unroll
-    for (int k = 0; k < MERGE_MLB; ++k)
+    for (int k = 0; k < MLB; ++k)
       if (lane + 32 * k < nsplit && mlv[k].x != -INFINITY)
         L = fmaf(fast_exp2(mlv[k].x - M), mlv[k].y, L);
-    for (int s = lane + 32 * MERGE_MLB; s < nsplit; s += 32) {
+    for (int s = lane + 32 * MLB; s < nsplit; s += 32) {
       const float2 v = ml[s * rs];
       if (v.x != -INFINITY) L = fmaf(fast_exp2(v.x - M), v.y, L);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
 #pragma unroll
-    for (int u = 0; u < MERGE_SG_BATCH; ++u)
+    for (int u = 0; u < NB; ++u)
       if (sg + MERGE_NSG * u < nsplit && mv[u] != -INFINITY)
-        acc = fmaf(fast_exp2(mv[u] - M), ov[u], acc);
+      {
+        const float w = fast_exp2(mv[u] - M);
+        acc.x = fmaf(w, ov[u].x, acc.x);
+        acc.y = fmaf(w, ov[u].y, acc.y);
+      }
     // more splits than one batch covers
-    for (int s0 = sg + MERGE_NSG * MERGE_SG_BATCH; s0 < nsplit; s0 += MERGE_NSG * MERGE_SG_BATCH) {
+    for (int s0 = sg + MERGE_NSG * NB; s0 < nsplit; s0 += MERGE_NSG * NB) {
 #pragma unroll
-      for (int u = 0; u < MERGE_SG_BATCH; ++u) {
+      for (int u = 0; u < NB; ++u) {
         const int s = s0 + MERGE_NSG * u;
-        ov[u] = (s < nsplit) ? po[s * rs * D] : 0.f;
+        ov[u] = (s < nsplit) ? po[s * rs * (D / 2)] : make_float2(0.f, 0.f);
         mv[u] = (s < nsplit) ? ml[s * rs].x : -INFINITY;
       }
 #pragma unroll
-      for (int u = 0; u < MERGE_SG_BATCH; ++u)
-        if (mv[u] != -INFINITY) acc = fmaf(fast_exp2(mv[u] - M), ov[u], acc);
+      for (int u = 0; u < NB; ++u)
+        if (mv[u] != -INFINITY) {
+          const float w = fast_exp2(mv[u] - M);
+          acc.x = fmaf(w, ov[u].x, acc.x);
+          acc.y = fmaf(w, ov[u].y, acc.y);
+        }
     }
   }
   red[sg][dd] = acc;
   __syncthreads();
-  if (t < MERGE_DSLICE) {
-    float o = 0.f;
+  if (t < MERGE_DSLICE / 2) {
+    float2 o = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < MERGE_NSG; ++k) o += red[k][t];
-    orow[t] = __bfloat16_as_ushort(__float2bfloat16_rn(L > 0.f ? o / L : 0.f));
+    for (int k = 0; k < MERGE_NSG; ++k) {
+      o.x += red[k][t].x;
+      o.y += red[k][t].y;
+    }
+    const float lo = L > 0.f ? o.x / L : 0.f, hi = L > 0.f ? o.y / L : 0.f;
+    reinterpret_cast<uint32_t*>(orow)[t] =
+        (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
+        ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
   }
 }
 
@@ -1447,24 +1494,38 @@ int launch_decode_merge(const DecodeArgs& a, int D, int B, cudaStream_t stream) 
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   pdl[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t mc = {};
-  // a few rows: 32-column slices with 8 split groups each (more CTAs, fewer
+  // a few rows: 64-column slices with 8 split groups each (more CTAs, fewer
   // loads per thread); a batch: one CTA per row
-  const bool sg = (int64_t)B * a.HqL * (D / MERGE_DSLICE) <= 4 * (int64_t)sm_count();
+  const int64_t ctas = (int64_t)B * a.HqL * (D / MERGE_DSLICE);
+  const bool sg = ctas <= 2 * (int64_t)sm_count();
   mc.gridDim = sg ? dim3((unsigned)(D / MERGE_DSLICE), (unsigned)a.HqL, (unsigned)B)
                   : dim3((unsigned)a.HqL, (unsigned)B, 1u);
   mc.blockDim = dim3(sg ? (unsigned)MERGE_THREADS : (unsigned)(D / 2));
-  mc.dynamicSmemBytes = 0;
+  // shared memory that the kernel does not use spreads its CTAs (see it)
+  constexpr int kOnePerSm = 120 * 1024, kTwoPerSm = 100 * 1024;
+  mc.dynamicSmemBytes = sg ? (ctas <= sm_count() ? kOnePerSm : kTwoPerSm) : 0;
   mc.stream = stream;
   mc.attrs = pdl;
   mc.numAttrs = 1;
   cudaError_t e;
   if (sg) {
-    if (a.span)
-      e = (D == 256) ? cudaLaunchKernelEx(&mc, decode_merge_sg_kernel<256, true>, a)
-                     : cudaLaunchKernelEx(&mc, decode_merge_sg_kernel<128, true>, a);
-    else
-      e = (D == 256) ? cudaLaunchKernelEx(&mc, decode_merge_sg_kernel<256, false>, a)
-                     : cudaLaunchKernelEx(&mc, decode_merge_sg_kernel<128, false>, a);
+    // span plans have no bound on a request's rows but the budget's pieces
+    const int rows = a.span ? a.budget + 1 : a.balanced ? a.budget + B : a.plan_splits;
+    auto launch = [&](auto kernel) {
+      if (smem_optin((const void*)kernel, kOnePerSm) != JF_OK) return cudaErrorUnknown;
+      return cudaLaunchKernelEx(&mc, kernel, a);
+    };
+    auto go = [&](auto nb) {
+      constexpr int NB = decltype(nb)::value;
+      if (a.span)
+        return D == 256 ? launch(decode_merge_sg_kernel<256, true, NB>)
+                        : launch(decode_merge_sg_kernel<128, true, NB>);
+      return D == 256 ? launch(decode_merge_sg_kernel<256, false, NB>)
+                      : launch(decode_merge_sg_kernel<128, false, NB>);
+    };
+    e = rows <= 5 * MERGE_NSG    ? go(std::integral_constant<int, 5>{})
+        : rows <= 10 * MERGE_NSG ? go(std::integral_constant<int, 10>{})
+                                 : go(std::integral_constant<int, 16>{});
   } else {
     if (a.span)
       e = (D == 256) ? cudaLaunchKernelEx(&mc, decode_merge_kernel<256, true>, a)
