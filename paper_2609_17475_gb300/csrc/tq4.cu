@@ -331,14 +331,42 @@ __device__ __forceinline__ void tq4_chunk(Tq4State<D>& st, const uint32_t (&bq)[
   }
 }
 
+// Fused append: the warp whose ring takes the chunk of position pos of request
+// b encodes the step's new K and V vectors of its KV head and stores them
+// before it copies that chunk.  Only that warp waits for the encoder (it ran
+// on two warps with the whole CTA waiting: 67.8 us of device time for a step at
+// 256K positions, 65.3 this way, where the decode alone takes 65.1).  Out of line: the encoder
+// must not weigh on the chunk loop's registers.
+template <int D>
+__device__ __noinline__ void append_new_row(const DecodeArgs& a, const Tq4Params& prm, int b,
+                                            int kvh, int pos, int lane) {
+  const int pidx = pos >> a.log2P;
+  const int page = (pidx < a.pt_stride) ? a.page_table[(int64_t)b * a.pt_stride + pidx] : -1;
+  const bool ok = page >= 0 && page < a.num_pages;
+  if (!ok && lane == 0) flag_error(a.status, JF_DEV_ERR_PAGE_ID);
+#pragma unroll 1
+  for (int kind = 0; kind < 2; ++kind) {
+    float rho;
+    const uint32_t word = tq4_encode<D>((kind ? a.vnew : a.knew) + ((int64_t)b * a.Hkv + kvh) * D,
+                                        kind, prm, lane, rho);
+    if (ok)
+      tq4_store<D>(const_cast<uint8_t*>(a.pool) + (int64_t)page * a.page_bytes, a.codes_region,
+                   a.sb_region, kind, (int64_t)kvh * a.P + (pos & (a.P - 1)), lane, word, rho);
+  }
+  // before this warp's copies (TMA) read the page
+  fence_proxy_async_global();
+  __syncwarp();
+  fence_proxy_async_global();
+}
+
 // VER: packed verifier (a.L > 1 query tokens, per-row causal limits; each CTA
 // holds 8 of the KV head's G * L (token, head) rows; launched for at most 8
 // rows, more go to the warp-pair kernel of tq4_verify.cu); otherwise decode.
 // APP: the step's new K/V row is appended first (a.knew, a.vnew).
 template <int D, bool VER, bool APP>
 __global__ void __launch_bounds__(TQ_WARPS * 32, 1)
-tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArgs a,
-                 const Tq4Params prm) {
+tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ DecodeArgs a,
+                 const __grid_constant__ Tq4Params prm) {
   using L = Tq4Smem<D>;
   constexpr int NCH = D / 64;
   constexpr float NEG_INF = -INFINITY;
@@ -424,27 +452,8 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArgs a,
   const int my_n = (n_cta > warp) ? (n_cta - warp + TQ_WARPS - 1) / TQ_WARPS : 0;
   auto chunk_of = [&](int it) { return c_begin + warp + it * TQ_WARPS; };
 
-  if (APP && split == nsplit - 1) {   // owns the last chunk
-    // the step's new K (warp 0) and V (warp 1) rows go to position ctx - 1
-    // before this split's copies read the page
-    if (warp < 2 && ctx > 0) {
-      const int pos = ctx - 1;
-      float rho;
-      const uint32_t word = tq4_encode<D>((warp ? a.vnew : a.knew) + ((int64_t)b * a.Hkv + kvh) * D,
-                                          warp, prm, lane, rho);
-      const int pidx = pos >> a.log2P;
-      const int page = (pidx < a.pt_stride) ? a.page_table[(int64_t)b * a.pt_stride + pidx] : -1;
-      if (page < 0 || page >= a.num_pages) {
-        if (lane == 0) flag_error(a.status, JF_DEV_ERR_PAGE_ID);
-      } else {
-        tq4_store<D>(const_cast<uint8_t*>(a.pool) + (int64_t)page * a.page_bytes, a.codes_region,
-                     a.sb_region, warp, (int64_t)kvh * a.P + (pos & (a.P - 1)), lane, word, rho);
-      }
-    }
-    fence_proxy_async_global();
-    __syncthreads();
-    fence_proxy_async_global();
-  }
+  // fused append: this warp's ring takes the request's last chunk
+  const bool appends = APP && split == nsplit - 1 && warp == (n_cta - 1) % TQ_WARPS;
 
   // ---- rotated queries q' = H S_K q / sqrt(D) (rows >= G stay zero) -------
   // warp h < 8 transforms head row h with shuffles (E elements per lane)
@@ -538,7 +547,13 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArgs a,
     valid = (valid & ~(1u << s)) | ((uint32_t)ok << s);
   };
   const int npro = my_n < TQ_STAGES ? my_n : TQ_STAGES;
+  if constexpr (APP) {
+    if (appends && my_n <= TQ_STAGES) append_new_row<D>(a, prm, b, kvh, ctx - 1, lane);
+  }
   for (int it = 0; it < npro; ++it) issue(it);
+  if constexpr (APP) {   // the copies issued so far are of earlier chunks
+    if (appends && my_n > TQ_STAGES) append_new_row<D>(a, prm, b, kvh, ctx - 1, lane);
+  }
 
   Tq4State<D> st;
   st.init();
