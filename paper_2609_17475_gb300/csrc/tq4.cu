@@ -363,7 +363,10 @@ __device__ __noinline__ void append_new_row(const DecodeArgs& a, const Tq4Params
 // holds 8 of the KV head's G * L (token, head) rows; launched for at most 8
 // rows, more go to the warp-pair kernel of tq4_verify.cu); otherwise decode.
 // APP: the step's new K/V row is appended first (a.knew, a.vnew).
-template <int D, bool VER, bool APP>
+// SPAN: batches under the span plan (decode.cuh): this CTA's piece of the
+// batch's chunks runs the same code once per request that it meets.  32
+// requests of 1K-64K positions (page 64): 397 us in whole-request pieces, 225 this way.
+template <int D, bool VER, bool APP, bool SPAN>
 __global__ void __launch_bounds__(TQ_WARPS * 32, 1)
 tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ DecodeArgs a,
                  const __grid_constant__ Tq4Params prm) {
@@ -410,50 +413,88 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
   }
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
 
-  int split, b, ctx, nch, cps, nsplit;
-  if (a.balanced) {
-    if (warp == 0) {
-      const BalPlan p = balanced_plan(a, (int)blockIdx.x, -1, lane);
-      if (lane == 0) {
-        misc[0] = p.b;
-        misc[1] = p.split;
-        misc[2] = p.nsplit;
-        misc[3] = p.cps;
-      }
-    }
-    __syncthreads();
-    b = misc[0];
-    split = misc[1];
-    nsplit = misc[2];
-    cps = misc[3];
-    if (b < 0) return;
-    ctx = checked_ctx(a, b, split);
-    nch = (ctx + DTOK - 1) / DTOK;
-  } else {
-    split = blockIdx.x;
-    b = blockIdx.z;
-    ctx = checked_ctx(a, b, split);
-    split_plan(ctx, a.num_splits, nch, cps, nsplit);
-  }
-  if (split >= nsplit) {
-    if (direct && split == 0) {
-      for (int i = threadIdx.x; i < rows * D; i += blockDim.x)
-        a.out[((int64_t)b * a.HqL + row_of(i / D)) * D + i % D] = 0;
-    }
-    return;
-  }
-  if (!aligned) {
+  if (SPAN && !aligned) {
     if (threadIdx.x == 0) flag_error(a.status, JF_DEV_ERR_LAYOUT);
     return;
   }
-  const int c_begin = split * cps;
-  const int c_end = min(c_begin + cps, nch);
+  // span plan: the places [pos, end) of the batch's sequence are this CTA's
+  long long pos = 0, end = 1;
+  if constexpr (SPAN) {
+    const long long T = span_total(a, lane);
+    const int W = span_width(T, a.budget);
+    pos = (long long)blockIdx.x * W;
+    end = min(pos + W, T);
+  }
+  uint32_t ph = 0;   // span plan: parity of the next wait on each stage (the ring runs on)
+  while (pos < end) {
+  int b, ctx, c_begin, c_end;
+  bool owns_last;            // holds the request's last chunk
+  int64_t prow0, prow_step;  // partial row of query row fr: prow0 + prow_step * fr
+  if constexpr (SPAN) {
+    const SpanHit h = span_find(a, pos, lane);
+    if (h.b < 0) break;
+    // offsets in the request's run: its first SPAN_HDR places hold no chunks
+    const int v0 = (int)(pos - h.start);
+    const int v1 = (int)(min(end, h.start + h.nch) - h.start);
+    b = h.b;
+    ctx = checked_ctx(a, b, v0);
+    c_begin = max(v0 - SPAN_HDR, 0);
+    c_end = max(v1 - SPAN_HDR, 0);
+    owns_last = v1 == h.nch;
+    prow0 = ((int64_t)blockIdx.x + b) * a.HqL;
+    prow_step = 1;
+    pos = h.start + v1;
+  } else {
+    pos = end;
+    int split, nch, cps, nsplit;
+    if (a.balanced) {
+      if (warp == 0) {
+        const BalPlan p = balanced_plan(a, (int)blockIdx.x, -1, lane);
+        if (lane == 0) {
+          misc[0] = p.b;
+          misc[1] = p.split;
+          misc[2] = p.nsplit;
+          misc[3] = p.cps;
+        }
+      }
+      __syncthreads();
+      b = misc[0];
+      split = misc[1];
+      nsplit = misc[2];
+      cps = misc[3];
+      if (b < 0) return;
+      ctx = checked_ctx(a, b, split);
+      nch = (ctx + DTOK - 1) / DTOK;
+    } else {
+      split = blockIdx.x;
+      b = blockIdx.z;
+      ctx = checked_ctx(a, b, split);
+      split_plan(ctx, a.num_splits, nch, cps, nsplit);
+    }
+    if (split >= nsplit) {
+      if (direct && split == 0) {
+        for (int i = threadIdx.x; i < rows * D; i += blockDim.x)
+          a.out[((int64_t)b * a.HqL + row_of(i / D)) * D + i % D] = 0;
+      }
+      return;
+    }
+    if (!aligned) {
+      if (threadIdx.x == 0) flag_error(a.status, JF_DEV_ERR_LAYOUT);
+      return;
+    }
+    c_begin = split * cps;
+    c_end = min(c_begin + cps, nch);
+    owns_last = split == nsplit - 1;
+    prow0 = a.balanced ? (int64_t)blockIdx.x * a.HqL
+                       : (int64_t)b * a.HqL * a.num_splits + blockIdx.x;
+    prow_step = a.balanced ? 1 : a.num_splits;
+  }
   const int n_cta = c_end - c_begin;
   const int my_n = (n_cta > warp) ? (n_cta - warp + TQ_WARPS - 1) / TQ_WARPS : 0;
   auto chunk_of = [&](int it) { return c_begin + warp + it * TQ_WARPS; };
 
   // fused append: this warp's ring takes the request's last chunk
-  const bool appends = APP && split == nsplit - 1 && warp == (n_cta - 1) % TQ_WARPS;
+  const bool appends = APP && owns_last && warp == (n_cta - 1) % TQ_WARPS;
 
   // ---- rotated queries q' = H S_K q / sqrt(D) (rows >= G stay zero) -------
   // warp h < 8 transforms head row h with shuffles (E elements per lane)
@@ -576,11 +617,12 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
 #pragma unroll 1
   for (int it = 0; it < my_n; ++it) {
     const int s = it % TQ_STAGES;
-    const uint32_t par = (it / TQ_STAGES) & 1;
+    const uint32_t par = SPAN ? (ph >> s) & 1u : (it / TQ_STAGES) & 1;
     if (!mbar_wait_bounded(&bars[warp * TQ_STAGES + s], par)) {
       if (lane == 0) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
       break;
     }
+    if constexpr (SPAN) ph ^= 1u << s;
     done = it + 1;
     const bool ok = (valid >> s) & 1u;
     const int tokbase = chunk_of(it) * DTOK;
@@ -599,9 +641,11 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
       issue(it + TQ_STAGES);
     }
   }
-  if (done < my_n) {
+  const bool gave_up = done < my_n;
+  if (gave_up) {
     for (int it = done; it < my_n && it < done + TQ_STAGES; ++it)
-      mbar_wait_bounded(&bars[warp * TQ_STAGES + it % TQ_STAGES], (it / TQ_STAGES) & 1, 1u << 16);
+      mbar_wait_bounded(&bars[warp * TQ_STAGES + it % TQ_STAGES],
+                        SPAN ? (ph >> (it % TQ_STAGES)) & 1u : (it / TQ_STAGES) & 1, 1u << 16);
   }
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 
@@ -697,8 +741,7 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
       else
         *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
     } else {
-      const int64_t row = a.balanced ? (int64_t)blockIdx.x * a.HqL + fr
-                                     : ((int64_t)b * a.HqL + fr) * a.num_splits + blockIdx.x;
+      const int64_t row = prow0 + prow_step * fr;
       float* dst = a.part_o + row * D + d0;
 #pragma unroll
       for (int e = 0; e < E; e += 4)
@@ -709,25 +752,34 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
       }
     }
   }
+  if constexpr (SPAN) {
+    // the next request's copies overwrite what this one's combine read here
+    fence_proxy_async_smem();
+    if (__syncthreads_or(gave_up ? 1 : 0)) return;   // a wait gave up (reported)
+  }
+  }
 }
 
-template <int D, bool VER, bool APP>
+template <int D, bool VER, bool APP, bool SPAN>
 static int launch_tq4_split(const cudaLaunchConfig_t& cfg0, const CUtensorMap& tmap,
                             const DecodeArgs& a, const Tq4Params& prm) {
-  if (smem_optin((const void*)tq4_split_kernel<D, VER, APP>, Tq4Smem<D>::TOTAL) != JF_OK)
+  if (smem_optin((const void*)tq4_split_kernel<D, VER, APP, SPAN>, Tq4Smem<D>::TOTAL) != JF_OK)
     return JF_ERR_CUDA;
   cudaLaunchConfig_t cfg = cfg0;
   cfg.dynamicSmemBytes = Tq4Smem<D>::TOTAL;
-  return cudaLaunchKernelEx(&cfg, tq4_split_kernel<D, VER, APP>, tmap, a, prm) == cudaSuccess
+  return cudaLaunchKernelEx(&cfg, tq4_split_kernel<D, VER, APP, SPAN>, tmap, a, prm) == cudaSuccess
              ? JF_OK : JF_ERR_CUDA;
 }
 
 template <int D>
 static int launch_tq4_split_any(const cudaLaunchConfig_t& cfg, const CUtensorMap& tmap,
                                 const DecodeArgs& a, const Tq4Params& prm) {
-  if (a.L > 1) return launch_tq4_split<D, true, false>(cfg, tmap, a, prm);
-  if (a.knew) return launch_tq4_split<D, false, true>(cfg, tmap, a, prm);
-  return launch_tq4_split<D, false, false>(cfg, tmap, a, prm);
+  if (a.L > 1) return launch_tq4_split<D, true, false, false>(cfg, tmap, a, prm);
+  if (a.span)
+    return a.knew ? launch_tq4_split<D, false, true, true>(cfg, tmap, a, prm)
+                  : launch_tq4_split<D, false, false, true>(cfg, tmap, a, prm);
+  if (a.knew) return launch_tq4_split<D, false, true, false>(cfg, tmap, a, prm);
+  return launch_tq4_split<D, false, false, false>(cfg, tmap, a, prm);
 }
 
 // packed verifier with more than 8 rows per KV head (tq4_verify.cu)
@@ -768,10 +820,13 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
   a.part_o = reinterpret_cast<float*>(ws + 256 + (rows * 8 + 255) / 256 * 256);
   a.num_splits = num_splits;
   a.plan_splits = num_splits;
-  a.span = 0;
   a.scale_log2 = softmax_scale * 1.4426950408889634f;
   a.B = batch;
-  a.balanced = (batch > 1 && batch <= 1024 && num_splits > 1) ? 1 : 0;
+  // batches share their splits: decode by the span plan, the verifier in
+  // whole-request pieces (as the affine decode)
+  const bool batch_plan = batch > 1 && batch <= 1024 && num_splits > 1;
+  a.span = (batch_plan && q_len == 1) ? 1 : 0;
+  a.balanced = (batch_plan && q_len > 1) ? 1 : 0;
   a.budget = 1;
   if (q_len > 1 && a.NT >= 2) {
     // warp pairs sharing the centroid lookups: ceil(NT / 3) CTAs per KV head
@@ -787,7 +842,11 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
     }
     return launch_tq4_verify_pairs(tmap, a, prm, g.D, batch, stream);
   }
-  if (a.balanced) {   // one CTA per SM in all
+  if (a.span) {   // one CTA per SM in all, within the workspace's rows
+    const int slots = (sm_count() + g.Hkv - 1) / g.Hkv;
+    const int64_t fit = (int64_t)batch * (num_splits - 1) + 1;
+    a.budget = (int)(fit < slots ? fit : slots);
+  } else if (a.balanced) {   // one CTA per SM in all
     const int slots = (sm_count() + g.Hkv * a.NT - 1) / (g.Hkv * a.NT);
     const int64_t fit = (int64_t)batch * num_splits - batch;
     const int64_t cap = fit < slots ? fit : slots;
@@ -797,7 +856,8 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   pdl[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = a.balanced ? dim3((unsigned)(a.budget + batch), (unsigned)(g.Hkv * a.NT), 1u)
+  cfg.gridDim = a.span ? dim3((unsigned)a.budget, (unsigned)g.Hkv, 1u)
+              : a.balanced ? dim3((unsigned)(a.budget + batch), (unsigned)(g.Hkv * a.NT), 1u)
                            : dim3((unsigned)num_splits, (unsigned)(g.Hkv * a.NT), (unsigned)batch);
   cfg.blockDim = dim3(TQ_WARPS * 32);
   cfg.stream = stream;
