@@ -33,7 +33,7 @@
 //               [D, D + 256); P_j (fp16) overwrites S columns already read.
 //               S over two tiles keeps the MMA at N = 128 (an N = 64 pair
 //               MMA takes as long as an N = 128 one).
-//   dequantize  (8 warps, TQ4 16) this CTA's halves of 64-position K/V tiles
+//   dequantize  (two sets of 8 warps) this CTA's halves of 64-position K/V tiles
 //               (4-bit codes -> fp16 integers through the mantissa of fp16
 //               1024, then x = code * scale + bias with one fused
 //               multiply-add) into 128B-swizzled buffers, one item (one
@@ -43,7 +43,9 @@
 //               V halves into four tile buffers (free once P V of the tile
 //               four back is done), each arriving on CTA 0's K-pair or V-tile
 //               barrier.
-//   softmax     (4 warps) one thread per row: Q row -> shared memory at the start;
+//   softmax     (4 warps) one thread per row: Q row -> shared memory at the start
+//               (only the MMA warp waits for that; the tiles start at once: 8
+//               chunks of 64 queries 244 -> 241 us);
 //               online softmax on S (tcgen05.ld), P back to TMEM as fp16
 //               over S columns already read (tcgen05.st) and an arrive on
 //               CTA 0's P barrier; the reference maximum moves (and O is
@@ -67,11 +69,11 @@
 //               to 1,196 us, 8 chunks of 64 queries after 4K-32K positions from
 //               354 to 269 us; with fewer instructions around each wait (mapped
 //               addresses, several polls a loop step, three-input maxima) to
-//               1,190 and 264 us.  What bounds it now: shared memory (the
+//               1,190 and 264 us.  What bounds the kernel: shared memory (the
 //               operands of S and P V, the rebuilt tiles' stores and the codes
-//               take ~2,030 of the ~3,200 cycles a tile pair and CTA takes) and
-//               issue slots (dequantization and softmax, 56 %); the tensor work
-//               alone is ~2,040 cycles.
+//               take ~2,030 of the ~2,900 cycles a tile pair and CTA takes) and
+//               issue slots (dequantization and softmax); the tensor work alone
+//               is ~2,040 cycles.
 // Within every 8 consecutive d the tiles store elements in the order
 // 0,4,1,5,2,6,3,7 (the pairs one 32-bit word of codes yields); Q uses the same
 // order, so Q K^T is unchanged, and the epilogue undoes it for O.  Q is
@@ -155,24 +157,22 @@ struct PfSmem {
 };
 
 // Warps: 0 MMA, 1 code copies, 2-3 idle, then dequantization and softmax, each
-// whole warpgroups.  TQ4 runs two sets of dequantization warps, one for the
-// even and one for the odd tiles: its centroid lookups wait on shared memory
-// (1,500 queries after 20,001 positions: 641 us with one set, 604 with two).
-// The affine conversion is bound by issue slots, and a second set only takes
-// them from the softmax (2,048 after 30,720: 1,189 against 1,257 us).
-// Two sets need a register split: every thread starts with LAUNCH_REGS, and
-// the softmax warpgroup's increase comes out of the others' decrease.
-template <int FMT>
+// whole warpgroups.  Two sets of dequantization warps, one for the even and one
+// for the odd tiles: a set alone waits on its barriers, conversions and (TQ4)
+// centroid lookups in turn (device time, 2,048 queries after 30,720 positions:
+// 1,120 us with one set, 1,076 with two, 1,107 with three; TQ4, 1,500 after
+// 20,001: 641 us of wall time with one, 604 with two).  They need a register
+// split: every thread starts with LAUNCH_REGS, and the softmax warpgroup's
+// increase comes out of the others' decrease.
 struct PfRoles {
-  static constexpr int SETS = FMT == JF_FMT_TQ4 ? 2 : 1;
+  static constexpr int SETS = 2;
   static constexpr int TMA_WARP = 1;
   static constexpr int DQ0 = 4;
   static constexpr int SM0 = DQ0 + SETS * PF_DQ_WARPS;
   static constexpr int THREADS = 32 * (SM0 + PF_SM_WARPS);
-  static constexpr bool SPLIT_REGS = SETS > 1;
   static constexpr int LAUNCH_REGS = 80, MMA_REGS = 48, DQ_REGS = 72, SM_REGS = 136;
-  static_assert(!SPLIT_REGS || 32 * (DQ0 * MMA_REGS + SETS * PF_DQ_WARPS * DQ_REGS +
-                                     PF_SM_WARPS * SM_REGS) <= THREADS * LAUNCH_REGS,
+  static_assert(32 * (DQ0 * MMA_REGS + SETS * PF_DQ_WARPS * DQ_REGS + PF_SM_WARPS * SM_REGS) <=
+                    THREADS * LAUNCH_REGS,
                 "register shares exceed the launch's");
   static_assert(SM0 % 4 == 0, "a softmax warp's id gives its TMEM lane quarter");
 };
@@ -244,11 +244,11 @@ __device__ __forceinline__ void sb_to_h2(uint32_t w, uint32_t& s2, uint32_t& b2)
 // FMT: JF_FMT_AFFINE4_G64, or JF_FMT_TQ4 (centroid table, rotated queries,
 // natural d order, partial outputs rotated back by the merge kernel)
 template <int D, int FMT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PfRoles<FMT>::THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PfRoles::THREADS, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                const __grid_constant__ PrefillArgs a) {
   using L = PfSmem<D, FMT>;
-  using R = PfRoles<FMT>;
+  using R = PfRoles;
   constexpr bool TQ = FMT == JF_FMT_TQ4;
   constexpr int NKB = D / 64;           // 64-wide d blocks
   constexpr int UPI = (D == 256) ? 2 : 1;   // 16-byte code units per dequant item
@@ -280,6 +280,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
   uint64_t* stg_full = bars + 18;                // [NST] a tile's code bytes have landed
   uint64_t* stg_free = bars + 18 + L::NST;       // [NST] ... and have been read
   int32_t* stg_n = reinterpret_cast<int32_t*>(bars + 18 + 2 * L::NST);   // [NST] positions of the tile that hold data
+  uint64_t* q_full = bars + 28;    // on CTA 0: both CTAs' Q rows stored
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_rank();
@@ -324,6 +325,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
       mbar_init(&pv_done[i], 1);
       mbar_init(&p_full[i], 2 * PF_SM_WARPS);
     }
+    mbar_init(q_full, 2 * PF_SM_WARPS);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&k_full[i], 2 * PF_DQ_WARPS);    // the 4 K warps of each CTA, twice
       mbar_init(&s_full[i], 1);
@@ -416,13 +418,15 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     }
     fence_proxy_async_smem();
   }
-  tc::fence_before();
-  __syncthreads();
-  tc::cluster_sync();   // both CTAs' Q rows are in shared memory before the first MMA
-  tc::fence_after();
+  // (the query rows are in shared memory before the first MMA; the other roles
+  // need not wait for them)
+  if (warp >= R::SM0) {
+    __syncwarp();
+    if (lane == 0) tc::arrive_cluster(q_full, 0);
+  }
 
   if (warp < R::DQ0) {
-  if constexpr (R::SPLIT_REGS) tc::setmaxnreg_dec<R::MMA_REGS>();
+  tc::setmaxnreg_dec<R::MMA_REGS>();
   if (warp == 0) {
     // ================= MMA issuer (CTA 0 of the pair) =================
     if (rank == 0) {
@@ -453,6 +457,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
       // instruction cache with the other roles.
       const int npairs = (ntiles + 1) >> 1;
       int jn = 0;   // next tile whose P V is due
+      ok = tc::wait_cluster(q_full, 0);
+      tc::fence_after();
       for (int i = 0; i <= npairs && ok; ++i) {
         if (i < npairs) {
           if (!tc::wait_cluster(&k_full[i & 1], (i >> 1) & 1)) { ok = false; break; }
@@ -512,7 +518,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     __syncwarp();
   }
   } else if (warp < R::SM0) {
-    if constexpr (R::SPLIT_REGS) tc::setmaxnreg_dec<R::DQ_REGS>();
+    tc::setmaxnreg_dec<R::DQ_REGS>();
     // ================= dequantization (this CTA's halves) =================
     // One item per thread: the code bytes of one position, 16 UPI of them.
     // K warp w: positions 32 rank + 8 w .. + 7 of the tile, whole rows (4 items
@@ -630,7 +636,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     }
     if (!ok && dt == 0) flag_error(a.status, JF_DEV_ERR_TIMEOUT);
   } else {
-    if constexpr (R::SPLIT_REGS) tc::setmaxnreg_inc<R::SM_REGS>();
+    tc::setmaxnreg_inc<R::SM_REGS>();
     // ================= softmax + epilogue (this CTA's 128 rows) =================
     // Rows past the chunk (padding) see every position: their Q rows are zero
     // and their outputs are never stored, and keeping them unmasked keeps the
@@ -918,15 +924,14 @@ static int launch_pf(const dim3& grid, const CUtensorMap* maps, const PrefillArg
                      cudaStream_t stream) {
   if (smem_optin((const void*)prefill_kernel<D, FMT>, PfSmem<D, FMT>::TOTAL) != JF_OK)
     return JF_ERR_CUDA;
-  if (PfRoles<FMT>::SPLIT_REGS) {   // a split of more than the launch has would wait forever
-    static const bool fits = [] {
-      cudaFuncAttributes fa;
-      return cudaFuncGetAttributes(&fa, (const void*)prefill_kernel<D, FMT>) == cudaSuccess &&
-             fa.numRegs >= PfRoles<FMT>::LAUNCH_REGS;
-    }();
-    if (!fits) return JF_ERR_CUDA;
-  }
-  prefill_kernel<D, FMT><<<grid, PfRoles<FMT>::THREADS, PfSmem<D, FMT>::TOTAL, stream>>>(maps[0], maps[1],
+  // a register split of more than the launch has would wait forever
+  static const bool fits = [] {
+    cudaFuncAttributes fa;
+    return cudaFuncGetAttributes(&fa, (const void*)prefill_kernel<D, FMT>) == cudaSuccess &&
+           fa.numRegs >= PfRoles::LAUNCH_REGS;
+  }();
+  if (!fits) return JF_ERR_CUDA;
+  prefill_kernel<D, FMT><<<grid, PfRoles::THREADS, PfSmem<D, FMT>::TOTAL, stream>>>(maps[0], maps[1],
                                                                           a);
   return cudaGetLastError() == cudaSuccess ? JF_OK : JF_ERR_CUDA;
 }
