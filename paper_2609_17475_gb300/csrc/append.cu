@@ -17,7 +17,7 @@ struct AppendArgs {
   int64_t page_bytes;
   int64_t codes_region;
   int64_t sb_region;
-  int32_t P;
+  int32_t P, log2P;   // P is a power of two
   int32_t Hkv;
   const int32_t* page_table;
   int32_t pt_stride;
@@ -52,8 +52,13 @@ __global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
   float xv[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   int32_t req = 0, pos = 0;
   if (active) {
-    row = vec / a.Hkv;
-    head = (int)(vec % a.Hkv);
+    if (vec <= 0x7FFFFFFF) {   // 64-bit division is ~100 instructions
+      row = (uint32_t)vec / (uint32_t)a.Hkv;
+      head = (int)((uint32_t)vec - (uint32_t)row * (uint32_t)a.Hkv);
+    } else {
+      row = vec / a.Hkv;
+      head = (int)(vec % a.Hkv);
+    }
     // the row's slot and its K and V elements are independent loads, issued
     // together; the page-table entry (which needs the slot) overlaps the
     // quantizer
@@ -62,9 +67,9 @@ __global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
     load8_bf16(a.k + (row * a.Hkv + head) * D + li * 8, xk);
     load8_bf16(a.v + (row * a.Hkv + head) * D + li * 8, xv);
   }
-  const bool slot_ok = req >= 0 && req < a.num_requests && pos >= 0 && pos / a.P < a.pt_stride;
+  const bool slot_ok = req >= 0 && req < a.num_requests && pos >= 0 && (pos >> a.log2P) < a.pt_stride;
   const int32_t page =
-      (active && slot_ok) ? a.page_table[(int64_t)req * a.pt_stride + pos / a.P] : -1;
+      (active && slot_ok) ? a.page_table[(int64_t)req * a.pt_stride + (pos >> a.log2P)] : -1;
   __nv_bfloat16 sk, bk, sv, bv;
   const uint32_t wk = quantize8(xk, sk, bk);
   const uint32_t wv = quantize8(xv, sv, bv);
@@ -80,8 +85,8 @@ __global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
     return;
   }
   uint8_t* const base = a.pool + (int64_t)page * a.page_bytes;
-  store_quantized<D>(base, a.codes_region, a.sb_region, a.P, head, pos % a.P, 0, li, wk, sk, bk);
-  store_quantized<D>(base, a.codes_region, a.sb_region, a.P, head, pos % a.P, 1, li, wv, sv, bv);
+  store_quantized<D>(base, a.codes_region, a.sb_region, a.P, head, pos & (a.P - 1), 0, li, wk, sk, bk);
+  store_quantized<D>(base, a.codes_region, a.sb_region, a.P, head, pos & (a.P - 1), 1, li, wv, sv, bv);
 }
 
 int launch_append(const Geom& g, const jf_kv_pool& pool, const int32_t* page_table,
@@ -95,6 +100,7 @@ int launch_append(const Geom& g, const jf_kv_pool& pool, const int32_t* page_tab
   a.codes_region = g.codes_region;
   a.sb_region = g.sb_region;
   a.P = g.P;
+  a.log2P = __builtin_ctz((unsigned)g.P);
   a.Hkv = g.Hkv;
   a.page_table = page_table;
   a.pt_stride = pt_stride;
