@@ -8,7 +8,16 @@
 namespace jfkv {
 
 constexpr int DTOK = 32;      // positions per pipeline stage (one chunk)
-constexpr int MIN_CPS = 16;   // minimum chunks per split (512 positions)
+// Minimum chunks per split, and places per piece of the span plan: short
+// contexts are bound by a warp's time on a chunk (~2.4 us), so they are cut
+// fine, as far as the merge's rows allow.  Device time of a call with 16 / 12 /
+// 6 / 4 / 2 chunks: 1,000 positions (24/4/256) 10.2 / 8.5 / 7.4 / 7.1 / 7.2 us;
+// 4,096 (8/2/128) 7.5 / 6.7 / 5.9 / 5.8 / 6.0; a step at 8,000 10.3 / 9.0 / 8.2 /
+// 8.2 / 8.2; a verifier call at 1,000 15.4 / - / 10.1 / 9.1 / 8.4.  Two requests
+// of 700 and 1,500 positions with 16 / 8 / 6 / 4 places: 13.3 / 13.1 / 10.2 / 13.0
+// us (finer pieces hold only places of a request's start).
+constexpr int MIN_CPS = 4;
+constexpr int SPAN_MIN = 6;
 constexpr float DTAU = 4.f;   // log2 headroom before the reference maximum moves
 
 struct DecodeArgs {
@@ -109,7 +118,7 @@ static __device__ BalPlan balanced_plan(const DecodeArgs& a, int x, int want_b, 
 // laid end to end (request 0 first), each request's run preceded by
 // SPAN_HDR places that stand for the cost of starting a segment (query
 // fragments, pipeline fill, the combine and its partial row), and cut into
-// pieces of W places, W = max(MIN_CPS, ceil(T / budget)), T the total: every
+// pieces of W places, W = max(SPAN_MIN, ceil(T / budget)), T the total: every
 // piece carries the same work however unequal the requests are, and a piece
 // that starts a request streams that many fewer chunks (32 measured best:
 // two requests 67.9 -> 64.6 us, 32 mixed requests 196-197 -> 191-193 us).  Piece x meets requests in
@@ -139,7 +148,7 @@ static __device__ long long span_total(const DecodeArgs& a, int lane) {
 
 __host__ __device__ inline int span_width(long long T, int budget) {
   long long w = (T + budget - 1) / (budget > 0 ? budget : 1);
-  return (int)(w < MIN_CPS ? MIN_CPS : w);
+  return (int)(w < SPAN_MIN ? SPAN_MIN : w);
 }
 
 struct SpanHit {
@@ -174,6 +183,15 @@ static __device__ SpanHit span_find(const DecodeArgs& a, long long pos, int lane
     base += __shfl_sync(0xffffffffu, incl, 31);
   }
   return SpanHit{-1, 0, 0};
+}
+
+// Partial rows of a piece that holds only places of a request's start: no
+// chunks, so their weight is zero (the merge then leaves their outputs alone).
+__device__ __forceinline__ void span_no_chunks(const DecodeArgs& a, int64_t row0, int rows) {
+  if ((int)threadIdx.x < rows) {
+    a.part_ml[(row0 + threadIdx.x) * 2 + 0] = -INFINITY;
+    a.part_ml[(row0 + threadIdx.x) * 2 + 1] = 0.f;
+  }
 }
 
 // Partial rows of request b under the span plan: rows row .. row + n - 1

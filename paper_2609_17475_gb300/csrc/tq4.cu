@@ -444,6 +444,10 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     prow0 = ((int64_t)blockIdx.x + b) * a.HqL;
     prow_step = 1;
     pos = h.start + v1;
+    if (c_end == 0) {
+      span_no_chunks(a, prow0 + kvh * a.G, rows);
+      continue;
+    }
   } else {
     pos = end;
     int split, nch, cps, nsplit;
