@@ -367,27 +367,61 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
                                     (((m & 7) ^ (r & 7)) << 4));
   };
   if (TQ && warp >= R::SM0) {
-    // rotated fp32 query row, natural d order (the centroid pairs are too)
-    const float* qrow = a.qrot + ((int64_t)(rq.row0 + q0 + qi) * a.Hq + kvh * a.G + r % a.G) * D;
-    float qmax = 0.f;
-    if (row_ok) {
-      for (int c4 = 0; c4 < D / 4; ++c4) {
-        const float4 w = *reinterpret_cast<const float4*>(qrow + 4 * c4);
-        qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(w.x), fabsf(w.y)), fmaxf(fabsf(w.z), fabsf(w.w))));
-      }
-    }
-    qmax *= fabsf(a.scale_log2);
-    qe = (qmax >= 16384.f) ? (ilogbf(qmax) - 13) : 0;
-    const float qs = ldexpf(a.scale_log2, -qe);
+    // Rotated fp32 query rows, natural d order (the centroid pairs are too).
+    // A load takes whole rows, 8 elements a lane: with a lane per row it took
+    // 16 bytes of 32 rows (a chunk of 64 queries and three more of 64 to 100 after
+    // 500 to 3,000 positions: 71 -> 62 us; 57 us with the epilogue's stores by
+    // rows, below; 1,500 queries at position 20,001: 571 -> 567).  The affine
+    // queries keep a lane per row: their rows are half as long, and by rows the
+    // long chunks ran 2-5 % slower.
+    const int my_q = row_ok ? qi * a.Hq + r % a.G : -1;   // row, from the tile's first
+    constexpr int LPR = D / 8, RPI = 32 / LPR;   // lanes per row, rows at a time
+    const float* qbase =
+        a.qrot + ((int64_t)(rq.row0 + q0) * a.Hq + kvh * a.G) * D + 8 * (lane % LPR);
+    float qmax = 0.f;                            // as far as this lane sees
 #pragma unroll 4
-    for (int m = 0; m < D / 8; ++m) {   // natural d order
+    for (int i = 0; i < 32 / RPI; ++i) {
+      const int rr = i * RPI + lane / LPR, row = quarter * 32 + rr, m = lane % LPR;
+      const int src = __shfl_sync(0xffffffffu, my_q, rr);
       float4 w0 = make_float4(0.f, 0.f, 0.f, 0.f), w1 = w0;
-      if (row_ok) {
-        w0 = *reinterpret_cast<const float4*>(qrow + 8 * m);
-        w1 = *reinterpret_cast<const float4*>(qrow + 8 * m + 4);
+      if (src >= 0) {
+        const float4* v = reinterpret_cast<const float4*>(qbase + (int64_t)src * D);
+        w0 = v[0];
+        w1 = v[1];
       }
-      *q_chunk(m) = make_uint4(pack_f16x2(w0.x * qs, w0.y * qs), pack_f16x2(w0.z * qs, w0.w * qs),
-                               pack_f16x2(w1.x * qs, w1.y * qs), pack_f16x2(w1.z * qs, w1.w * qs));
+      qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(w0.x), fabsf(w0.y)), fmaxf(fabsf(w0.z), fabsf(w0.w))));
+      qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(w1.x), fabsf(w1.y)), fmaxf(fabsf(w1.z), fabsf(w1.w))));
+      const float qs = a.scale_log2;
+      *reinterpret_cast<uint4*>(sQ + (m >> 3) * (PF_BM * 128) + row * 128 +
+                                (((m & 7) ^ (row & 7)) << 4)) =
+          make_uint4(pack_f16x2(w0.x * qs, w0.y * qs), pack_f16x2(w0.z * qs, w0.w * qs),
+                     pack_f16x2(w1.x * qs, w1.y * qs), pack_f16x2(w1.z * qs, w1.w * qs));
+    }
+    // values past fp16's comfort (or not numbers): each row with its own power
+    // of two, a lane per row
+    if (__any_sync(0xffffffffu, !(qmax * fabsf(a.scale_log2) < 16384.f))) {
+      __syncwarp();
+      const float* qrow = a.qrot + ((int64_t)(rq.row0 + q0 + qi) * a.Hq + kvh * a.G + r % a.G) * D;
+      qmax = 0.f;
+      if (row_ok) {
+        for (int c4 = 0; c4 < D / 4; ++c4) {
+          const float4 w = *reinterpret_cast<const float4*>(qrow + 4 * c4);
+          qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(w.x), fabsf(w.y)), fmaxf(fabsf(w.z), fabsf(w.w))));
+        }
+      }
+      qmax *= fabsf(a.scale_log2);
+      qe = (qmax >= 16384.f) ? (ilogbf(qmax) - 13) : 0;
+      const float qs = ldexpf(a.scale_log2, -qe);
+#pragma unroll 4
+      for (int m = 0; m < D / 8; ++m) {   // natural d order
+        float4 w0 = make_float4(0.f, 0.f, 0.f, 0.f), w1 = w0;
+        if (row_ok) {
+          w0 = *reinterpret_cast<const float4*>(qrow + 8 * m);
+          w1 = *reinterpret_cast<const float4*>(qrow + 8 * m + 4);
+        }
+        *q_chunk(m) = make_uint4(pack_f16x2(w0.x * qs, w0.y * qs), pack_f16x2(w0.z * qs, w0.w * qs),
+                                 pack_f16x2(w1.x * qs, w1.y * qs), pack_f16x2(w1.z * qs, w1.w * qs));
+      }
     }
     fence_proxy_async_smem();
   } else if (warp >= R::SM0) {
@@ -760,38 +794,64 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
         a.part_ml[prow * 2 + 0] = m_ref;
         a.part_ml[prow * 2 + 1] = l;
       }
+      if constexpr (TQ) {
+        // Partial rows leave through this warp's quarter of the Q buffer (its
+        // last reader is done), half a row at a time, chunks swizzled by the
+        // row: a store instruction then writes whole half rows.
+        constexpr int ROWB = 2 * D, CH = ROWB / 16;   // bytes and 16-byte chunks of half a row
+        uint8_t* const slab = sQ + quarter * 32 * ROWB;
+        const unsigned long long dst0 = row_ok ? (unsigned long long)prow_o : 0ull;
 #pragma unroll 1
-      for (int c0 = 0; c0 < D; c0 += 32) {
-        uint32_t o[32];
-        tc::ld32(tO + c0 + lane_off, o);
-        tc::wait_ld();
-        if (row_ok && split) {
+        for (int hf = 0; hf < 2; ++hf) {
+#pragma unroll 1
+          for (int c0 = 0; c0 < D / 2; c0 += 32) {
+            uint32_t o[32];
+            tc::ld32(tO + hf * (D / 2) + c0 + lane_off, o);
+            tc::wait_ld();
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float* v = reinterpret_cast<const float*>(o + 8 * k);
-            float4* dst = reinterpret_cast<float4*>(prow_o + c0 + 8 * k);
-            if constexpr (TQ) {
-              dst[0] = make_float4(v[0], v[1], v[2], v[3]);
-              dst[1] = make_float4(v[4], v[5], v[6], v[7]);
-            } else {
+            for (int k = 0; k < 8; ++k)
+              *reinterpret_cast<uint4*>(slab + lane * ROWB + (((c0 / 4 + k) ^ (lane & 7)) << 4)) =
+                  make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+          }
+          __syncwarp();
+#pragma unroll 4
+          for (int i = 0; i < CH; ++i) {   // 32 / CH rows at a time
+            const int rr = i * (32 / CH) + lane / CH, ch = lane % CH;
+            const uint4 w = *reinterpret_cast<const uint4*>(slab + rr * ROWB + ((ch ^ (rr & 7)) << 4));
+            const unsigned long long dst = __shfl_sync(0xffffffffu, dst0, rr);
+            if (dst) *reinterpret_cast<uint4*>(dst + (unsigned)(hf * ROWB + 16 * ch)) = w;
+          }
+          __syncwarp();
+        }
+      } else {
+#pragma unroll 1
+        for (int c0 = 0; c0 < D; c0 += 32) {
+          uint32_t o[32];
+          tc::ld32(tO + c0 + lane_off, o);
+          tc::wait_ld();
+          if (row_ok && split) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float* v = reinterpret_cast<const float*>(o + 8 * k);
+              float4* dst = reinterpret_cast<float4*>(prow_o + c0 + 8 * k);
               dst[0] = make_float4(v[0], v[2], v[4], v[6]);
               dst[1] = make_float4(v[1], v[3], v[5], v[7]);
             }
-          }
-        } else if (row_ok) {
+          } else if (row_ok) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float* v = reinterpret_cast<const float*>(o + 8 * k);
-            uint4 w;
-            w.x = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[0] * inv)) |
-                  ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2] * inv)) << 16);
-            w.y = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[4] * inv)) |
-                  ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[6] * inv)) << 16);
-            w.z = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[1] * inv)) |
-                  ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[3] * inv)) << 16);
-            w.w = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[5] * inv)) |
-                  ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[7] * inv)) << 16);
-            *reinterpret_cast<uint4*>(orow + c0 + 8 * k) = w;
+            for (int k = 0; k < 4; ++k) {
+              const float* v = reinterpret_cast<const float*>(o + 8 * k);
+              uint4 w;
+              w.x = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[0] * inv)) |
+                    ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2] * inv)) << 16);
+              w.y = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[4] * inv)) |
+                    ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[6] * inv)) << 16);
+              w.z = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[1] * inv)) |
+                    ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[3] * inv)) << 16);
+              w.w = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[5] * inv)) |
+                    ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[7] * inv)) << 16);
+              *reinterpret_cast<uint4*>(orow + c0 + 8 * k) = w;
+            }
           }
         }
       }
