@@ -30,7 +30,8 @@ int launch_tq4_decode(const Geom&, const jf_kv_pool&, const CUtensorMap&, const 
 int decode_box_rows();
 int prefill_box_rows(bool v);
 int launch_prefill_batch(const Geom&, const jf_kv_pool&, const CUtensorMap*,
-                         const int32_t* const*, const int32_t*, const int32_t*, const void*, const int64_t*, int32_t, int32_t, float,
+                         const int32_t* const*, const int32_t*, const int32_t*, const void*,
+                         const int64_t*, int32_t, int32_t, float,
                          int32_t, void*, void*, cudaStream_t, int32_t, int64_t,
                          const Tq4Params*);
 size_t prefill_workspace_bytes(int64_t rows, int64_t Hq, int64_t D, int64_t S, int fmt);

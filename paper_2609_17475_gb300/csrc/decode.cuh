@@ -114,15 +114,15 @@ static __device__ BalPlan balanced_plan(const DecodeArgs& a, int x, int want_b, 
   return p;
 }
 
-// Span plan (batches of the affine decode).  The chunks of all requests are
+// Span plan (decode batches of either format).  The chunks of all requests are
 // laid end to end (request 0 first), each request's run preceded by
 // SPAN_HDR places that stand for the cost of starting a segment (query
 // fragments, pipeline fill, the combine and its partial row), and cut into
 // pieces of W places, W = max(SPAN_MIN, ceil(T / budget)), T the total: every
 // piece carries the same work however unequal the requests are, and a piece
 // that starts a request streams that many fewer chunks (32 measured best:
-// two requests 67.9 -> 64.6 us, 32 mixed requests 196-197 -> 191-193 us).  Piece x meets requests in
-// segments; the segment of request b is one split whose partial rows are
+// two requests 67.9 -> 64.6 us, 32 mixed requests 196-197 -> 191-193 us).
+// Piece x meets requests in segments; the segment of request b is one split whose partial rows are
 // (x + b) * HqL + hq (along the sequence every piece or request boundary
 // advances x + b, so the numbers never repeat, and a request's rows are
 // contiguous: x0_b + b .. x1_b + b).  The workspace holds B * num_splits
