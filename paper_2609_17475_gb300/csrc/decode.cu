@@ -1159,8 +1159,8 @@ decode_span_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArgs a)
 // Its CTAs are placed while the split kernel's leave, as many on an SM as fit,
 // and so crowded onto the first SMs to fall free: 24 heads x 8 slices of 32
 // sat on a quarter of the chip.  Now 24 x 4 slices of 64, and the launch asks
-// for as much (unused) shared memory as lets one of them on an SM, or two where
-// there are more than SMs.  Device time of a call: 256K positions 52.0 -> 50.5
+// for as much (unused) shared memory as lets one of them on an SM, or two, four
+// or eight where there are more.  Device time of a call: 256K positions 52.0 -> 50.5
 // us (TQ4 65.1 -> 64.2), fused step at 35,841 positions 15.7 -> 14.7 us, two
 // requests of 196,608 + 131,072 64.6 -> 63.2 us.  Slices of 32 with two on an SM
 // had given 50.8, 64.5, 15.0 and 64.8 us.
@@ -1494,16 +1494,25 @@ int launch_decode_merge(const DecodeArgs& a, int D, int B, cudaStream_t stream) 
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   pdl[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t mc = {};
-  // a few rows: 64-column slices with 8 split groups each (more CTAs, fewer
-  // loads per thread); a batch: one CTA per row
+  // up to two rows per SM: 64-column slices with 8 split groups each (more CTAs,
+  // fewer loads per thread); more rows: one CTA per row.  Device time of a call
+  // with a CTA per row and with slices, 24/4/256: 4 requests of 9K to 40K positions
+  // 30.8 and 28.9 us, 6 37.5 and 36.0, 8 41.6 and 39.7, 12 of 1K to 20K (288 rows)
+  // 30.5 and 30.4; past the line (384 rows of 128) 29.4 and 29.5.
   const int64_t ctas = (int64_t)B * a.HqL * (D / MERGE_DSLICE);
-  const bool sg = ctas <= 2 * (int64_t)sm_count();
+  const bool sg = (int64_t)B * a.HqL <= 2 * (int64_t)sm_count();
   mc.gridDim = sg ? dim3((unsigned)(D / MERGE_DSLICE), (unsigned)a.HqL, (unsigned)B)
                   : dim3((unsigned)a.HqL, (unsigned)B, 1u);
   mc.blockDim = dim3(sg ? (unsigned)MERGE_THREADS : (unsigned)(D / 2));
-  // shared memory that the kernel does not use spreads its CTAs (see it)
-  constexpr int kOnePerSm = 120 * 1024, kTwoPerSm = 100 * 1024;
-  mc.dynamicSmemBytes = sg ? (ctas <= sm_count() ? kOnePerSm : kTwoPerSm) : 0;
+  // shared memory that the kernel does not use spreads its CTAs (see it): room
+  // for one, two, four or eight of them on an SM
+  const int64_t sms = sm_count();
+  constexpr int kOnePerSm = 120 * 1024;
+  mc.dynamicSmemBytes = !sg                ? 0
+                        : ctas <= sms     ? kOnePerSm
+                        : ctas <= 2 * sms ? 100 * 1024
+                        : ctas <= 4 * sms ? 50 * 1024
+                                          : 24 * 1024;
   mc.stream = stream;
   mc.attrs = pdl;
   mc.numAttrs = 1;
