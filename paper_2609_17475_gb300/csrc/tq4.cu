@@ -545,7 +545,10 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
       bq[ch][s][0] = pack_f16x2(v.x * qmul, v.y * qmul);
       bq[ch][s][1] = pack_f16x2(v.z * qmul, v.w * qmul);
     }
-  __syncthreads();   // the query buffer lies in the stage rings the copies fill
+  // the query buffer lies in the stage rings: a barrier alone does not order its
+  // reads and writes before the copies (async proxy) that fill them
+  fence_proxy_async_smem();
+  __syncthreads();
 
   // ---- page ids and TMA producer (as in the affine decode) ---------------
   auto load_pages = [&](int blk) -> int {

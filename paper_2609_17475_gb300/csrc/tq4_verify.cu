@@ -413,7 +413,10 @@ tq4_verify_pair_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArg
     qsm[i] = make_uint4(pack_f16x2(x0.x * qmul, x0.y * qmul), pack_f16x2(x0.z * qmul, x0.w * qmul),
                         pack_f16x2(x1.x * qmul, x1.y * qmul), pack_f16x2(x1.z * qmul, x1.w * qmul));
   }
-  __syncthreads();   // the rotated rows lie in the rings the copies fill
+  // the rotated rows lie in the rings: a barrier alone does not order their
+  // reads and writes before the copies (async proxy) that fill them
+  fence_proxy_async_smem();
+  __syncthreads();
 
   // ---- page ids and the pair's TMA producer (as in verify.cu) -------------
   auto load_pages = [&](int blk) -> int {
