@@ -1116,7 +1116,9 @@ decode_span_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArgs a)
       }
     }
     // one CTA-wide answer (and the barrier after which a span plan's next
-    // split may reuse the rings and query fragments)
+    // split may reuse the rings and query fragments; its copies go through the
+    // async proxy, which the barrier alone does not order after the accesses above)
+    fence_proxy_async_smem();
     return __syncthreads_or(gave_up ? 1 : 0) == 0;
   };
 

@@ -19,6 +19,7 @@ HANDOVER = re.compile(r"fence_proxy_async_smem\(\);\s*(?:return |if \()?__syncth
     ("tq4_verify.cu", "tq4_verify_pair_kernel(", "qsm[i] = make_uint4(", "issue(it);"),
     # span plan: the combined output of a request, before the next one's copies
     ("tq4.cu", "tq4_split_kernel(", "x[e] = qbuf[", "template <int D, bool VER"),
+    ("decode.cu", "decode_span_kernel(", "+ w * WCODES) + h * SROW + d", "run_split(h.b, ctx"),
 ])
 def test_rings_are_fenced_before_copies_refill_them(file, kernel, last_access, first_copy):
     text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, file)).read())
