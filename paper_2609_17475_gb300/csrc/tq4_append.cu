@@ -112,7 +112,9 @@ tq4_append_general_kernel(const __grid_constant__ Tq4AppendArgs a, const __grid_
 // (the outer two run on); its word is the float threshold (in units of rho)
 // that lies in it or within 1/64 cell of it, rounded to a multiple of 16 ulps,
 // with the number of thresholds below the cell in the low 4 bits (a huge
-// threshold where there is none).  False if a cell would need two.
+// threshold where there is none).  A threshold at or next to zero is taken as
+// 2^-40, well inside the margin below: the count's place among the bits of a
+// zero would make them those of a NaN.  False if a cell would need two.
 constexpr int TQ_CELLS = 65;
 struct Tq4Lut {
   uint32_t w[TQ_CELLS];
@@ -130,6 +132,7 @@ static bool tq4_make_lut(const Tq4Params& p, Tq4Lut* lut) {
       thr = p.tq[below];
       if (below < 14 && p.tq[below + 1] <= hi) return false;
     }
+    if (std::fabs(thr) < 0x1p-40f) thr = 0x1p-40f;
     uint32_t b;
     std::memcpy(&b, &thr, 4);
     lut->w[i] = ((b - below + 8) & ~15u) | below;
