@@ -34,15 +34,18 @@ __device__ __forceinline__ uint32_t quantize8(const float (&x)[8], __nv_bfloat16
     // exceeds k + 1/2 by more than half an ulp (a tie rounds down, k + 1/2
     // being even).  Only the threshold next to the quotient is in doubt, an
     // approximate quotient finds it, and near it a - scale (k + 1/2) is exact
-    // in one fma (scale (k + 1/2) has 13 bits), so no division is needed.
+    // in one fma (scale (k + 1/2) has 13 bits), so no division is needed.  (At
+    // the group's maximum, 15.06 scale at most, k may come out 15, which no
+    // quotient exceeds by half.)  A NaN element exceeds no threshold: the
+    // maximum drops it, k is 0 and its comparison false.
     // 2,048 rows of 24/4/256: 8.2 -> 5.6 us of device time (5.1 with the append
     // kernel's index arithmetic in 32 bits), 8,192 rows 28.4 -> 20.3 (18.5).
     const float inv = __frcp_rn(scale), s24 = scale * 0x1p-24f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const float a = __fsub_rn(x[i], bias);
-      const float t = __fadd_rn(fminf(__fmaf_rn(a, inv, -0.5f), 14.f), 12582912.f);
-      const float k5 = __fadd_rn(__fsub_rn(t, 12582912.f), 0.5f);   // k + 1/2, k = 0 .. 14
+      const float t = __fadd_rn(fmaxf(__fmaf_rn(a, inv, -0.5f), -0.5f), 12582912.f);
+      const float k5 = __fadd_rn(__fsub_rn(t, 12582912.f), 0.5f);   // k + 1/2, k = 0 .. 15
       // half an ulp of k + 1/2, times scale
       const float half = __fmul_rn(s24, __uint_as_float(__float_as_uint(k5) & 0x7F800000u));
       uint32_t c = __float_as_uint(t);                              // low bits: k
