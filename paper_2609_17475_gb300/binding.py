@@ -208,8 +208,7 @@ class Tq4Codec:
         for j in range(head_dim):
             c.signs_k[j] = int(sk[j])
             c.signs_v[j] = int(sv[j])
-        self._c = c
-        self._p = ctypes.pointer(c)
+        self._c = c   # no ctypes pointer to it: an object that holds one is not copied or pickled
 
 
 @dataclasses.dataclass
@@ -252,7 +251,7 @@ class KVPool:
         p = _Pool(data.data_ptr(), data.shape[0], self.page_size, self.num_kv_heads,
                   self.head_dim, self.group_size, self.format)
         if self.codec is not None:
-            p.tq4 = self.codec._p
+            p.tq4 = ctypes.pointer(self.codec._c)
         return p
 
 
