@@ -147,15 +147,19 @@ def _check(fn: str, status: int) -> None:
 # the smallest calls run for less time than that on the GPU.  So: addresses and
 # the stream are plain integers (the C signatures convert them), the current
 # stream's handle is read without building a torch.cuda.Stream (0.2 against
-# 3.1 us), and a tensor is checked and its address read in one step.  A decode
-# call took 16.5 us of host time, now 9.9, an append 13.9, now 7.5.
-_raw_stream = torch._C._cuda_getCurrentRawStream
-_device = torch._C._cuda_getDevice
+# 3.1 us; a torch without these two functions, one built without CUDA among
+# them, has the package imported all the same and takes the public call), and a
+# tensor is checked and its address read in one step.  A decode call took 16.5 us
+# of host time, now 9.9, an append 13.9, now 7.5.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
 _I32, _BF16, _U8 = torch.int32, torch.bfloat16, torch.uint8
 
 
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is None or _device is None:
+            return torch.cuda.current_stream().cuda_stream
         return _raw_stream(_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
