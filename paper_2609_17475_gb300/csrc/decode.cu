@@ -32,7 +32,8 @@
 // split partial (m, l, O) to the workspace, or straight to the output when
 // num_splits == 1.
 //
-// Kernel 2 (merge).  CTAs over (32-wide d slice, query head, request) combine:
+// Kernel 2 (merge).  CTAs over (64-wide d slice, query head, request), or one per
+// (query head, request) where there are more of those than fit at once, combine:
 //   o = sum_s 2^{m_s - m*} O_s / sum_s 2^{m_s - m*} l_s.
 #include <cmath>
 #include <cfloat>
@@ -1161,8 +1162,8 @@ decode_span_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArgs a)
 // Its CTAs are placed while the split kernel's leave, as many on an SM as fit,
 // and so crowded onto the first SMs to fall free: 24 heads x 8 slices of 32
 // sat on a quarter of the chip.  Now 24 x 4 slices of 64, and the launch asks
-// for as much (unused) shared memory as lets one of them on an SM, or two, four
-// or eight where there are more.  Device time of a call: 256K positions 52.0 -> 50.5
+// for as much (unused) shared memory as lets one of them on an SM, or two, or four
+// where there are more (then as many as the registers allow).  Device time of a call: 256K positions 52.0 -> 50.5
 // us (TQ4 65.1 -> 64.2), fused step at 35,841 positions 15.7 -> 14.7 us, two
 // requests of 196,608 + 131,072 64.6 -> 63.2 us.  Slices of 32 with two on an SM
 // had given 50.8, 64.5, 15.0 and 64.8 us.
@@ -1186,9 +1187,14 @@ __device__ __forceinline__ float ld_here(const float* p) {
 
 // NB: splits per thread in a batch, the smallest of 5, 10 and 16 that holds
 // the plan's splits (38 of them need 5; loads past the plan still cost their
-// issue).
+// issue).  Registers hold a batch, so an SM takes six, four or two CTAs.
+constexpr int merge_nb(int rows) {
+  return rows <= 5 * MERGE_NSG ? 5 : rows <= 10 * MERGE_NSG ? 10 : 16;
+}
+constexpr int merge_per_sm(int nb) { return nb == 5 ? 6 : nb == 10 ? 4 : 2; }
+
 template <int D, bool SPAN, int NB>
-__global__ void __launch_bounds__(MERGE_THREADS) decode_merge_sg_kernel(const DecodeArgs a) {
+__global__ void __launch_bounds__(MERGE_THREADS, merge_per_sm(NB)) decode_merge_sg_kernel(const DecodeArgs a) {
   // SPAN: partial rows of the span plan.  A template parameter: the span
   // branch in the single-request instance, though never taken, had slowed
   // the 256K call by ~1.2 us.
@@ -1496,18 +1502,26 @@ int launch_decode_merge(const DecodeArgs& a, int D, int B, cudaStream_t stream) 
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   pdl[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t mc = {};
-  // up to two rows per SM: 64-column slices with 8 split groups each (more CTAs,
-  // fewer loads per thread); more rows: one CTA per row.  Device time of a call
-  // with a CTA per row and with slices, 24/4/256: 4 requests of 9K to 40K positions
-  // 30.8 and 28.9 us, 6 37.5 and 36.0, 8 41.6 and 39.7, 12 of 1K to 20K (288 rows)
-  // 30.5 and 30.4; past the line (384 rows of 128) 29.4 and 29.5.
+  // span plans have no bound on a request's rows but the budget's pieces
+  const int rows = a.span ? a.budget + 1 : a.balanced ? a.budget + B : a.plan_splits;
+  const int nb = merge_nb(rows);
+  // Up to two rows per SM, and as long as all their CTAs fit on the chip at
+  // once: 64-column slices with 8 split groups each (more CTAs, fewer loads per
+  // thread); more: one CTA per row.  Device time of a call with a CTA per row and
+  // with slices, 24/4/256 (six CTAs an SM): 4 requests of 9K to 40K positions 30.8
+  // and 28.9 us, 6 37.5 and 36.0, 8 41.6 and 39.7; 12 of 500 to 12K, 1,152 CTAs for
+  // 912 places, 22.7 and 23.5.  12/2/256 (four): 12 requests, 576 CTAs, 17.9 and
+  // 17.0; 24, 1,152, 20.0 and 22.3.  One KV head (two): 38 of 8/1/128, 608 CTAs,
+  // 15.6 and 17.8; 49 of 6/1/256, 1,176, 23.5 and 30.0; a verifier's 16 x 3 tokens
+  // of 6/1/256, 1,152, 18.0 and 24.9.
   const int64_t ctas = (int64_t)B * a.HqL * (D / MERGE_DSLICE);
-  const bool sg = (int64_t)B * a.HqL <= 2 * (int64_t)sm_count();
+  const bool sg = (int64_t)B * a.HqL <= 2 * (int64_t)sm_count() &&
+                  ctas <= (int64_t)merge_per_sm(nb) * sm_count();
   mc.gridDim = sg ? dim3((unsigned)(D / MERGE_DSLICE), (unsigned)a.HqL, (unsigned)B)
                   : dim3((unsigned)a.HqL, (unsigned)B, 1u);
   mc.blockDim = dim3(sg ? (unsigned)MERGE_THREADS : (unsigned)(D / 2));
   // shared memory that the kernel does not use spreads its CTAs (see it): room
-  // for one, two, four or eight of them on an SM
+  // for one, two, four or as many as the registers allow on an SM
   const int64_t sms = sm_count();
   constexpr int kOnePerSm = 120 * 1024;
   mc.dynamicSmemBytes = !sg                ? 0
@@ -1520,8 +1534,6 @@ int launch_decode_merge(const DecodeArgs& a, int D, int B, cudaStream_t stream) 
   mc.numAttrs = 1;
   cudaError_t e;
   if (sg) {
-    // span plans have no bound on a request's rows but the budget's pieces
-    const int rows = a.span ? a.budget + 1 : a.balanced ? a.budget + B : a.plan_splits;
     auto launch = [&](auto kernel) {
       if (smem_optin((const void*)kernel, kOnePerSm) != JF_OK) return cudaErrorUnknown;
       return cudaLaunchKernelEx(&mc, kernel, a);
@@ -1534,9 +1546,9 @@ int launch_decode_merge(const DecodeArgs& a, int D, int B, cudaStream_t stream) 
       return D == 256 ? launch(decode_merge_sg_kernel<256, false, NB>)
                       : launch(decode_merge_sg_kernel<128, false, NB>);
     };
-    e = rows <= 5 * MERGE_NSG    ? go(std::integral_constant<int, 5>{})
-        : rows <= 10 * MERGE_NSG ? go(std::integral_constant<int, 10>{})
-                                 : go(std::integral_constant<int, 16>{});
+    e = nb == 5    ? go(std::integral_constant<int, 5>{})
+        : nb == 10 ? go(std::integral_constant<int, 10>{})
+                   : go(std::integral_constant<int, 16>{});
   } else {
     if (a.span)
       e = (D == 256) ? cudaLaunchKernelEx(&mc, decode_merge_kernel<256, true>, a)
