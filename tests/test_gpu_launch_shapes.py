@@ -48,3 +48,13 @@ def test_sliced_merge_fits_on_the_chip_at_once(fmt, Hq, Hkv, D, q_len):
         if sliced:
             assert merge.ctas <= merge.resident, (B, merge)
     assert kinds == {True, False}
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(64, 16, 128), (24, 6, 256), (12, 3, 256), (10, 5, 128),
+                                      (24, 12, 128), (28, 7, 128), (24, 4, 256), (200, 200, 128)])
+def test_tq4_batch_pieces_fit_on_the_chip_at_once(Hq, Hkv, D):
+    """A TQ4 batch's pieces are equal, so one more than fit at once makes two
+    rounds of them: 172.6 against 104.9 us (16 KV heads, 160 pieces)."""
+    for B in (2, 8, 24):
+        (split,) = [x for x in _batch(jf.JF_FMT_TQ4, Hq, Hkv, D, B) if "tq4_split" in x.name]
+        assert split.ctas <= max(split.resident, Hkv), (B, split)
