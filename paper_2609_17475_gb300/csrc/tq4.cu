@@ -331,32 +331,38 @@ __device__ __forceinline__ void tq4_chunk(Tq4State<D>& st, const uint32_t (&bq)[
   }
 }
 
-// Fused append: the warp whose ring takes the chunk of position pos of request
-// b encodes the step's new K and V vectors of its KV head and stores them
-// before it copies that chunk.  Only that warp waits for the encoder (it ran
-// on two warps with the whole CTA waiting: 67.8 us of device time for a step at
-// 256K positions, 65.3 this way, where the decode alone takes 65.1).  Out of line: the encoder
-// must not weigh on the chunk loop's registers.
+// Fused append: encodes the step's new K (kind 0) or V (1) vector of a KV head
+// and stores it at position pos of request b.  The warp whose ring takes that
+// position's chunk does K and the next warp V; the first waits for the second
+// before it copies the chunk, the others not at all.  Device time of a step at
+// 600 / 18,000 / 262,144 positions (24/4/256): 12.4 / 13.5 / 69.8 us with two
+// warps and the whole CTA waiting, 14.0 / 15.3 / 65.7 with both vectors on the
+// one warp, 12.3 / 13.3 / 64.9 this way.  Out of line: the encoder must not
+// weigh on the chunk loop's registers.
+constexpr int APPEND_BAR = 1;   // named barrier of the two warps
 template <int D>
-__device__ __noinline__ void append_new_row(const DecodeArgs& a, const Tq4Params& prm, int b,
-                                            int kvh, int pos, int lane) {
+__device__ __noinline__ void append_new_vector(const DecodeArgs& a, const Tq4Params& prm, int b,
+                                               int kvh, int kind, int pos, int lane) {
   const int pidx = pos >> a.log2P;
   const int page = (pidx < a.pt_stride) ? a.page_table[(int64_t)b * a.pt_stride + pidx] : -1;
   const bool ok = page >= 0 && page < a.num_pages;
   if (!ok && lane == 0) flag_error(a.status, JF_DEV_ERR_PAGE_ID);
-#pragma unroll 1
-  for (int kind = 0; kind < 2; ++kind) {
-    float rho;
-    const uint32_t word = tq4_encode<D>((kind ? a.vnew : a.knew) + ((int64_t)b * a.Hkv + kvh) * D,
-                                        kind, prm, lane, rho);
-    if (ok)
-      tq4_store<D>(const_cast<uint8_t*>(a.pool) + (int64_t)page * a.page_bytes, a.codes_region,
-                   a.sb_region, kind, (int64_t)kvh * a.P + (pos & (a.P - 1)), lane, word, rho);
-  }
-  // before this warp's copies (TMA) read the page
+  float rho;
+  const uint32_t word = tq4_encode<D>((kind ? a.vnew : a.knew) + ((int64_t)b * a.Hkv + kvh) * D,
+                                      kind, prm, lane, rho);
+  if (ok)
+    tq4_store<D>(const_cast<uint8_t*>(a.pool) + (int64_t)page * a.page_bytes, a.codes_region,
+                 a.sb_region, kind, (int64_t)kvh * a.P + (pos & (a.P - 1)), lane, word, rho);
+  // before the first warp's copies (TMA) read the page: fenced on both sides of
+  // the barrier
   fence_proxy_async_global();
   __syncwarp();
-  fence_proxy_async_global();
+  if (kind) {
+    asm volatile("bar.arrive %0, 64;\n" ::"n"(APPEND_BAR) : "memory");
+  } else {
+    asm volatile("bar.sync %0, 64;\n" ::"n"(APPEND_BAR) : "memory");
+    fence_proxy_async_global();
+  }
 }
 
 // VER: packed verifier (a.L > 1 query tokens, per-row causal limits; each CTA
@@ -497,8 +503,10 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
   const int my_n = (n_cta > warp) ? (n_cta - warp + TQ_WARPS - 1) / TQ_WARPS : 0;
   auto chunk_of = [&](int it) { return c_begin + warp + it * TQ_WARPS; };
 
-  // fused append: this warp's ring takes the request's last chunk
-  const bool appends = APP && owns_last && warp == (n_cta - 1) % TQ_WARPS;
+  // fused append: this warp's ring takes the request's last chunk, or the ring
+  // of the one before does
+  const bool encodes_k = APP && owns_last && warp == (n_cta - 1) % TQ_WARPS;
+  const bool encodes_v = APP && owns_last && warp == n_cta % TQ_WARPS;
 
   // ---- rotated queries q' = H S_K q / sqrt(D) (rows >= G stay zero) -------
   // warp h < 8 transforms head row h with shuffles (E elements per lane)
@@ -596,11 +604,13 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
   };
   const int npro = my_n < TQ_STAGES ? my_n : TQ_STAGES;
   if constexpr (APP) {
-    if (appends && my_n <= TQ_STAGES) append_new_row<D>(a, prm, b, kvh, ctx - 1, lane);
+    if (encodes_k && my_n <= TQ_STAGES)
+      append_new_vector<D>(a, prm, b, kvh, 0, ctx - 1, lane);
   }
   for (int it = 0; it < npro; ++it) issue(it);
   if constexpr (APP) {   // the copies issued so far are of earlier chunks
-    if (appends && my_n > TQ_STAGES) append_new_row<D>(a, prm, b, kvh, ctx - 1, lane);
+    if (encodes_k && my_n > TQ_STAGES) append_new_vector<D>(a, prm, b, kvh, 0, ctx - 1, lane);
+    if (encodes_v) append_new_vector<D>(a, prm, b, kvh, 1, ctx - 1, lane);
   }
 
   Tq4State<D> st;
