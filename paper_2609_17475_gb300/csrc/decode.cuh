@@ -114,7 +114,8 @@ static __device__ BalPlan balanced_plan(const DecodeArgs& a, int x, int want_b, 
   return p;
 }
 
-// Span plan (decode batches of either format).  The chunks of all requests are
+// Span plan (decode batches; few requests of the TQ4 format keep the plan
+// above, see launch_tq4_decode).  The chunks of all requests are
 // laid end to end (request 0 first), each request's run preceded by
 // SPAN_HDR places that stand for the cost of starting a segment (query
 // fragments, pipeline fill, the combine and its partial row), and cut into

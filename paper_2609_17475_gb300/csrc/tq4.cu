@@ -371,7 +371,8 @@ __device__ __noinline__ void append_new_vector(const DecodeArgs& a, const Tq4Par
 // APP: the step's new K/V row is appended first (a.knew, a.vnew).
 // SPAN: batches under the span plan (decode.cuh): this CTA's piece of the
 // batch's chunks runs the same code once per request that it meets.  32
-// requests of 1K-64K positions (page 64): 397 us in whole-request pieces, 225 this way.
+// requests of 1K-64K positions (page 64): 397 us in whole-request pieces, 225 this
+// way.  (Few requests keep whole-request pieces, see launch_tq4_decode.)
 template <int D, bool VER, bool APP, bool SPAN>
 __global__ void __launch_bounds__(TQ_WARPS * 32, 1)
 tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ DecodeArgs a,
@@ -839,11 +840,21 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
   a.plan_splits = num_splits;
   a.scale_log2 = softmax_scale * 1.4426950408889634f;
   a.B = batch;
-  // batches share their splits: decode by the span plan, the verifier in
-  // whole-request pieces (as the affine decode)
+  // Batches share their splits: decode by the span plan, the verifier in
+  // whole-request pieces (as the affine decode), and so is a decode with 19 SMs
+  // or more for each request and KV head.  There the pieces come out about
+  // equal, and a span's piece that ends one request and begins the next pays
+  // two queries, combines and (fused step) encoders for few chunks.  Device time
+  // of a step in spans and in whole-request pieces: 24/4/256 with 11,407 + 4,719
+  // positions 18.1 and 16.1 us, 8/2/128 9,913 + 4,815 12.2 and 11.2, 8/1/128
+  // 34,106 + 68,576 13.9 and 11.8; of a decode, 24/4/256 803 + 1,060 11.7 and 11.0,
+  // 77,216 + 21,264 33.1 and 33.2, 196,608 + 131,072 80.3 and 81.9.  With 15 SMs
+  // (five requests of 8/2/128, 536 to 22,128) 11.2 and 15.0, with 5 (24/6/256)
+  // 31.6 and 38.0.
   const bool batch_plan = batch > 1 && batch <= 1024 && num_splits > 1;
-  a.span = (batch_plan && q_len == 1) ? 1 : 0;
-  a.balanced = (batch_plan && q_len > 1) ? 1 : 0;
+  const bool whole = q_len > 1 || 19 * (int64_t)batch * g.Hkv <= sm_count();
+  a.span = (batch_plan && !whole) ? 1 : 0;
+  a.balanced = (batch_plan && whole) ? 1 : 0;
   a.budget = 1;
   if (q_len > 1 && a.NT >= 2) {
     // warp pairs sharing the centroid lookups: ceil(NT / 3) CTAs per KV head
@@ -859,15 +870,19 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
     }
     return launch_tq4_verify_pairs(tmap, a, prm, g.D, batch, stream);
   }
-  if (a.span) {
+  if (batch_plan && q_len == 1) {
     // One CTA per SM in all, within the workspace's rows.  Rounded down: the
     // pieces are equal, so one that finds no SM free makes a second round.  24
     // requests of 1K to 20K positions with the quotient rounded up and down: 172.6
     // and 104.9 us (64/16/128), 90.0 and 58.0 (24/6/256), 113.2 and 70.4
     // (28/7/128); 2, 4 and 8 KV heads divide the SMs.
     const int slots = sm_count() / g.Hkv > 1 ? sm_count() / g.Hkv : 1;
-    const int64_t fit = (int64_t)batch * (num_splits - 1) + 1;
+    const int64_t fit = a.span ? (int64_t)batch * (num_splits - 1) + 1
+                               : (int64_t)batch * num_splits;
     a.budget = (int)(fit < slots ? fit : slots);
+    // whole-request pieces are at most budget + batch - 1 (each request's last
+    // one rounds up)
+    if (a.balanced) a.budget = a.budget - batch + 1 > 1 ? a.budget - batch + 1 : 1;
   } else if (a.balanced) {   // one CTA per SM in all
     const int slots = (sm_count() + g.Hkv * a.NT - 1) / (g.Hkv * a.NT);
     const int64_t fit = (int64_t)batch * num_splits - batch;
@@ -879,7 +894,7 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
   pdl[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = a.span ? dim3((unsigned)a.budget, (unsigned)g.Hkv, 1u)
-              : a.balanced ? dim3((unsigned)(a.budget + batch), (unsigned)(g.Hkv * a.NT), 1u)
+              : a.balanced ? dim3((unsigned)(a.budget + batch - 1), (unsigned)(g.Hkv * a.NT), 1u)
                            : dim3((unsigned)num_splits, (unsigned)(g.Hkv * a.NT), (unsigned)batch);
   cfg.blockDim = dim3(TQ_WARPS * 32);
   cfg.stream = stream;

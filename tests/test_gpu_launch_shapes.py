@@ -58,3 +58,16 @@ def test_tq4_batch_pieces_fit_on_the_chip_at_once(Hq, Hkv, D):
     for B in (2, 8, 24):
         (split,) = [x for x in _batch(jf.JF_FMT_TQ4, Hq, Hkv, D, B) if "tq4_split" in x.name]
         assert split.ctas <= max(split.resident, Hkv), (B, split)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(6, 1, 256), (8, 2, 128), (12, 3, 256), (24, 4, 256),
+                                      (32, 8, 128)])
+def test_tq4_few_requests_take_whole_request_pieces(Hq, Hkv, D):
+    """With 19 SMs or more for each request and KV head; spans from there on."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for B in range(2, 12):
+        (split,) = [x for x in _batch(jf.JF_FMT_TQ4, Hq, Hkv, D, B) if "tq4_split" in x.name]
+        spans = f"ILi{D}ELb0ELb0ELb1E" in split.name
+        assert spans or f"ILi{D}ELb0ELb0ELb0E" in split.name, split
+        assert spans == (19 * B * Hkv > sms), (B, split)
+        assert split.ctas <= split.resident, (B, split)
