@@ -241,6 +241,21 @@ __device__ __forceinline__ void sb_to_h2(uint32_t w, uint32_t& s2, uint32_t& b2)
   b2 = pack_f16x2(b, b);
 }
 
+// Loads that stay where they are written, so that a batch of them is in flight
+// before the first is used.
+__device__ __forceinline__ float4 ld_here(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_here(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];\n"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 // FMT: JF_FMT_AFFINE4_G64, or JF_FMT_TQ4 (centroid table, rotated queries,
 // natural d order, partial outputs rotated back by the merge kernel)
 template <int D, int FMT>
@@ -360,6 +375,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
   const int r = quarter * 32 + lane;
   const bool row_ok = r < rows;
   const int qi = row_ok ? r / a.G : 0;
+  const int wrows = min(32, max(0, rows - quarter * 32));   // this warp's rows that hold queries
   const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
   int qe = 0;                                  // per-row power of two kept out of fp16
   auto q_chunk = [&](int m) -> uint4* {
@@ -374,28 +390,41 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     // rows, below; 1,500 queries at position 20,001: 571 -> 567).  The affine
     // queries keep a lane per row: their rows are half as long, and by rows the
     // long chunks ran 2-5 % slower.
-    const int my_q = row_ok ? qi * a.Hq + r % a.G : -1;   // row, from the tile's first
+    // The loads of QB steps are issued together (as branches of one loop, each
+    // waited for its own: twenty queries of 24/4/256 at position 0, 25.1 us of
+    // device time, 19.2 now; eight of 32/8/128 16.8 and 14.1).
+    const int my_q = qi * a.Hq + r % a.G;        // row, from the tile's first
     constexpr int LPR = D / 8, RPI = 32 / LPR;   // lanes per row, rows at a time
+    constexpr int QB = 4;
     const float* qbase =
         a.qrot + ((int64_t)(rq.row0 + q0) * a.Hq + kvh * a.G) * D + 8 * (lane % LPR);
     float qmax = 0.f;                            // as far as this lane sees
-#pragma unroll 4
-    for (int i = 0; i < 32 / RPI; ++i) {
-      const int rr = i * RPI + lane / LPR, row = quarter * 32 + rr, m = lane % LPR;
-      const int src = __shfl_sync(0xffffffffu, my_q, rr);
-      float4 w0 = make_float4(0.f, 0.f, 0.f, 0.f), w1 = w0;
-      if (src >= 0) {
-        const float4* v = reinterpret_cast<const float4*>(qbase + (int64_t)src * D);
-        w0 = v[0];
-        w1 = v[1];
+#pragma unroll 1
+    for (int i0 = 0; i0 < 32 / RPI; i0 += QB) {
+      float4 w[QB][2];
+#pragma unroll
+      for (int u = 0; u < QB; ++u) {
+        w[u][0] = w[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int rr = (i0 + u) * RPI + lane / LPR;
+        const int src = __shfl_sync(0xffffffffu, my_q, rr);
+        if (rr < wrows) {
+          const float4* v = reinterpret_cast<const float4*>(qbase + (int64_t)src * D);
+          w[u][0] = ld_here(v);
+          w[u][1] = ld_here(v + 1);
+        }
       }
-      qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(w0.x), fabsf(w0.y)), fmaxf(fabsf(w0.z), fabsf(w0.w))));
-      qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(w1.x), fabsf(w1.y)), fmaxf(fabsf(w1.z), fabsf(w1.w))));
-      const float qs = a.scale_log2;
-      *reinterpret_cast<uint4*>(sQ + (m >> 3) * (PF_BM * 128) + row * 128 +
-                                (((m & 7) ^ (row & 7)) << 4)) =
-          make_uint4(pack_f16x2(w0.x * qs, w0.y * qs), pack_f16x2(w0.z * qs, w0.w * qs),
-                     pack_f16x2(w1.x * qs, w1.y * qs), pack_f16x2(w1.z * qs, w1.w * qs));
+#pragma unroll
+      for (int u = 0; u < QB; ++u) {
+        const float4 w0 = w[u][0], w1 = w[u][1];
+        const int row = quarter * 32 + (i0 + u) * RPI + lane / LPR, m = lane % LPR;
+        qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(w0.x), fabsf(w0.y)), fmaxf(fabsf(w0.z), fabsf(w0.w))));
+        qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(w1.x), fabsf(w1.y)), fmaxf(fabsf(w1.z), fabsf(w1.w))));
+        const float qs = a.scale_log2;
+        *reinterpret_cast<uint4*>(sQ + (m >> 3) * (PF_BM * 128) + row * 128 +
+                                  (((m & 7) ^ (row & 7)) << 4)) =
+            make_uint4(pack_f16x2(w0.x * qs, w0.y * qs), pack_f16x2(w0.z * qs, w0.w * qs),
+                       pack_f16x2(w1.x * qs, w1.y * qs), pack_f16x2(w1.z * qs, w1.w * qs));
+      }
     }
     // values past fp16's comfort (or not numbers): each row with its own power
     // of two, a lane per row
@@ -425,31 +454,41 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     }
     fence_proxy_async_smem();
   } else if (warp >= R::SM0) {
+    // One pass with the common scale, QB loads at a time; only a row with values
+    // past fp16's comfort is read again, scaled by a power of two of its own.
+    // (Two passes, the first for the maximum, read 512 bytes of each row twice
+    // through an L1 that the staging ring leaves 28 KB: eight queries of 24/4/256 at
+    // position 0, 15.2 us of device time, 11.1 now; 64 queries 17.3 and 12.7.)
     const uint16_t* qrow = rq.q + ((int64_t)(q0 + qi) * a.Hq + kvh * a.G + r % a.G) * D;
+    constexpr int QB = 8;
     float qmax = 0.f;
-    if (row_ok) {
-      for (int c8 = 0; c8 < D / 8; ++c8) {
-        const uint4 w = *reinterpret_cast<const uint4*>(qrow + 8 * c8);
-        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+    auto load_rows = [&](float qs) {
+#pragma unroll 1
+      for (int m0 = 0; m0 < D / 8; m0 += QB) {
+        uint4 w[QB];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          qmax = fmaxf(qmax, fmaxf(fabsf(bf16lo_to_f32(ws[k])), fabsf(bf16hi_to_f32(ws[k]))));
+        for (int u = 0; u < QB; ++u) {
+          w[u] = make_uint4(0, 0, 0, 0);
+          if (row_ok) w[u] = ld_here(reinterpret_cast<const uint4*>(qrow + 8 * (m0 + u)));
+        }
+#pragma unroll
+        for (int u = 0; u < QB; ++u) {
+          const float e0 = bf16lo_to_f32(w[u].x), e1 = bf16hi_to_f32(w[u].x);
+          const float e2 = bf16lo_to_f32(w[u].y), e3 = bf16hi_to_f32(w[u].y);
+          const float e4 = bf16lo_to_f32(w[u].z), e5 = bf16hi_to_f32(w[u].z);
+          const float e6 = bf16lo_to_f32(w[u].w), e7 = bf16hi_to_f32(w[u].w);
+          qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(e0), fabsf(e1)), fmaxf(fabsf(e2), fabsf(e3))));
+          qmax = fmaxf(qmax, fmaxf(fmaxf(fabsf(e4), fabsf(e5)), fmaxf(fabsf(e6), fabsf(e7))));
+          *q_chunk(m0 + u) =
+              make_uint4(pack_f16x2(e0 * qs, e4 * qs), pack_f16x2(e1 * qs, e5 * qs),
+                         pack_f16x2(e2 * qs, e6 * qs), pack_f16x2(e3 * qs, e7 * qs));
+        }
       }
-    }
+    };
+    load_rows(a.scale_log2);
     qmax *= a.scale_log2;
     qe = (qmax >= 16384.f) ? (ilogbf(qmax) - 13) : 0;
-    const float qs = ldexpf(a.scale_log2, -qe);
-#pragma unroll 4
-    for (int m = 0; m < D / 8; ++m) {
-      uint4 w = make_uint4(0, 0, 0, 0);
-      if (row_ok) w = *reinterpret_cast<const uint4*>(qrow + 8 * m);
-      const float e0 = bf16lo_to_f32(w.x) * qs, e1 = bf16hi_to_f32(w.x) * qs;
-      const float e2 = bf16lo_to_f32(w.y) * qs, e3 = bf16hi_to_f32(w.y) * qs;
-      const float e4 = bf16lo_to_f32(w.z) * qs, e5 = bf16hi_to_f32(w.z) * qs;
-      const float e6 = bf16lo_to_f32(w.w) * qs, e7 = bf16hi_to_f32(w.w) * qs;
-      *q_chunk(m) = make_uint4(pack_f16x2(e0, e4), pack_f16x2(e1, e5), pack_f16x2(e2, e6),
-                               pack_f16x2(e3, e7));
-    }
+    if (__any_sync(0xffffffffu, qe != 0)) load_rows(ldexpf(a.scale_log2, -qe));
     fence_proxy_async_smem();
   }
   // (the query rows are in shared memory before the first MMA; the other roles
@@ -794,7 +833,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
         a.part_ml[prow * 2 + 0] = m_ref;
         a.part_ml[prow * 2 + 1] = l;
       }
-      if constexpr (TQ) {
+      if (TQ && wrows > 0) {
         // Partial rows leave through this warp's quarter of the Q buffer (its
         // last reader is done), half a row at a time, chunks swizzled by the
         // row: a store instruction then writes whole half rows.
@@ -815,7 +854,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
           }
           __syncwarp();
 #pragma unroll 4
-          for (int i = 0; i < CH; ++i) {   // 32 / CH rows at a time
+          for (int i = 0; i * (32 / CH) < wrows; ++i) {   // 32 / CH rows at a time
             const int rr = i * (32 / CH) + lane / CH, ch = lane % CH;
             const uint4 w = *reinterpret_cast<const uint4*>(slab + rr * ROWB + ((ch ^ (rr & 7)) << 4));
             const unsigned long long dst = __shfl_sync(0xffffffffu, dst0, rr);
@@ -823,7 +862,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
           }
           __syncwarp();
         }
-      } else {
+      }
+      if constexpr (!TQ) {
 #pragma unroll 1
         for (int c0 = 0; c0 < D; c0 += 32) {
           uint32_t o[32];
