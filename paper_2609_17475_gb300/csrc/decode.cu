@@ -1648,7 +1648,16 @@ int launch_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& tmap
   a.B = batch;
   const int nw = decode_warps(batch, num_splits, g.Hkv, a.NT);
   const int per_sm = 12 / nw;   // split CTAs resident per SM
-  const int slots = (per_sm * sm_count() + g.Hkv * a.NT - 1) / (g.Hkv * a.NT);
+  // Decode rounds them down: one split more than the SMs take makes a second
+  // round.  With 16 KV heads, 10 splits each on 152 SMs and 9: one request of
+  // 64/16/128 with 1,600 / 5,000 / 40,000 positions 9.5 / 12.7 / 38.9 and 6.4 /
+  // 8.4 / 23.1 us, 12 of 24/12/128 44.9 and 29.1.  The verifier's 6-warp CTAs
+  // share an SM unevenly and go on as others end; there rounding up is the
+  // faster (12 of 64/16/128 with two tokens 107.8 and 121.3).
+  const int per_head = g.Hkv * a.NT;
+  const int down = per_sm * sm_count() / per_head;
+  const int slots = q_len > 1 ? (per_sm * sm_count() + per_head - 1) / per_head
+                              : (down > 1 ? down : 1);
   // per-request plans: one CTA wave (12-warp CTAs) or the caller's cap
   a.plan_splits = (nw == 12 && num_splits > slots) ? slots : num_splits;
   // Batches of up to BAL_MAX_B requests size their splits for the whole
@@ -1672,8 +1681,8 @@ int launch_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& tmap
   if (q_len > 1 && a.NT >= 2) {
     // packed verifier with more than 8 rows per KV head: warp pairs share the
     // unpacking (verify.cu), one 8-warp CTA per SM, ncta CTAs per KV head
-    const int per_head = g.Hkv * verify_pair_ctas(a.NT);
-    const int vslots = sm_count() / per_head > 1 ? sm_count() / per_head : 1;
+    const int pair_ctas = g.Hkv * verify_pair_ctas(a.NT);
+    const int vslots = sm_count() / pair_ctas > 1 ? sm_count() / pair_ctas : 1;
     a.plan_splits = num_splits < vslots ? num_splits : vslots;
     if (a.balanced) {
       const int64_t fit = (int64_t)batch * num_splits - batch;

@@ -480,7 +480,7 @@ tq4_split_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
       split = blockIdx.x;
       b = blockIdx.z;
       ctx = checked_ctx(a, b, split);
-      split_plan(ctx, a.num_splits, nch, cps, nsplit);
+      split_plan(ctx, a.plan_splits, nch, cps, nsplit);
     }
     if (split >= nsplit) {
       if (direct && split == 0) {
@@ -837,7 +837,11 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
   a.part_ml = reinterpret_cast<float*>(ws + 256);
   a.part_o = reinterpret_cast<float*>(ws + 256 + (rows * 8 + 255) / 256 * 256);
   a.num_splits = num_splits;
-  a.plan_splits = num_splits;
+  // a single request's decode: one split per SM at most, as the affine decode
+  // (64/16/128 with 1,600 / 5,000 / 40,000 positions: 11.7 / 15.4 / 48.6 us with 10
+  // splits on 9.5 SMs a head, 7.7 / 9.6 / 28.6 with 9)
+  const int slots = sm_count() / g.Hkv > 1 ? sm_count() / g.Hkv : 1;
+  a.plan_splits = (batch == 1 && q_len == 1 && num_splits > slots) ? slots : num_splits;
   a.scale_log2 = softmax_scale * 1.4426950408889634f;
   a.B = batch;
   // Batches share their splits: decode by the span plan, the verifier in
@@ -876,7 +880,6 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
     // requests of 1K to 20K positions with the quotient rounded up and down: 172.6
     // and 104.9 us (64/16/128), 90.0 and 58.0 (24/6/256), 113.2 and 70.4
     // (28/7/128); 2, 4 and 8 KV heads divide the SMs.
-    const int slots = sm_count() / g.Hkv > 1 ? sm_count() / g.Hkv : 1;
     const int64_t fit = a.span ? (int64_t)batch * (num_splits - 1) + 1
                                : (int64_t)batch * num_splits;
     a.budget = (int)(fit < slots ? fit : slots);
@@ -884,9 +887,9 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
     // one rounds up)
     if (a.balanced) a.budget = a.budget - batch + 1 > 1 ? a.budget - batch + 1 : 1;
   } else if (a.balanced) {   // one CTA per SM in all
-    const int slots = (sm_count() + g.Hkv * a.NT - 1) / (g.Hkv * a.NT);
+    const int up = (sm_count() + g.Hkv * a.NT - 1) / (g.Hkv * a.NT);
     const int64_t fit = (int64_t)batch * num_splits - batch;
-    const int64_t cap = fit < slots ? fit : slots;
+    const int64_t cap = fit < up ? fit : up;
     a.budget = (int)(cap - batch / 2 > 1 ? cap - batch / 2 : 1);
   }
   cudaLaunchAttribute pdl[1];
@@ -895,7 +898,7 @@ int launch_tq4_decode(const Geom& g, const jf_kv_pool& pool, const CUtensorMap& 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = a.span ? dim3((unsigned)a.budget, (unsigned)g.Hkv, 1u)
               : a.balanced ? dim3((unsigned)(a.budget + batch - 1), (unsigned)(g.Hkv * a.NT), 1u)
-                           : dim3((unsigned)num_splits, (unsigned)(g.Hkv * a.NT), (unsigned)batch);
+                           : dim3((unsigned)a.plan_splits, (unsigned)(g.Hkv * a.NT), (unsigned)batch);
   cfg.blockDim = dim3(TQ_WARPS * 32);
   cfg.stream = stream;
   cfg.attrs = pdl;

@@ -71,3 +71,13 @@ def test_tq4_few_requests_take_whole_request_pieces(Hq, Hkv, D):
         assert spans or f"ILi{D}ELb0ELb0ELb0E" in split.name, split
         assert spans == (19 * B * Hkv > sms), (B, split)
         assert split.ctas <= split.resident, (B, split)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(64, 16, 128), (24, 6, 256), (12, 3, 256), (10, 5, 128),
+                                      (24, 12, 128), (28, 7, 128), (24, 4, 256), (200, 200, 128)])
+@pytest.mark.parametrize("fmt", [jf.JF_FMT_AFFINE4_G64, jf.JF_FMT_TQ4])
+def test_decode_splits_fit_on_the_chip_at_once(fmt, Hq, Hkv, D):
+    """One request and (affine) batches, at the default split counts."""
+    for B in (1, 2, 12):
+        (split,) = [x for x in _batch(fmt, Hq, Hkv, D, B) if "merge" not in x.name]
+        assert split.ctas <= max(split.resident, Hkv), (B, split)
