@@ -1185,11 +1185,13 @@ __device__ __forceinline__ float ld_here(const float* p) {
   return v;
 }
 
-// NB: splits per thread in a batch, the smallest of 5, 10 and 16 that holds
-// the plan's splits (38 of them need 5; loads past the plan still cost their
-// issue).  Registers hold a batch, so an SM takes six, four or two CTAs.
+// NB: splits per thread in a batch, the smallest of 5, 10 and 19 that holds
+// the plan's splits: 38, 76 and 152 of them with four, two and one KV heads on 152
+// SMs (loads past the plan still cost their issue: ~0.1 us).  A second batch is
+// a second memory round trip: one request of 6/1/256 at 60,000 positions, 145 splits,
+// 12.5 us with batches of 16, 11.3 with 19.  Registers hold a batch, so an SM takes six, four or two CTAs.
 constexpr int merge_nb(int rows) {
-  return rows <= 5 * MERGE_NSG ? 5 : rows <= 10 * MERGE_NSG ? 10 : 16;
+  return rows <= 5 * MERGE_NSG ? 5 : rows <= 10 * MERGE_NSG ? 10 : 19;
 }
 constexpr int merge_per_sm(int nb) { return nb == 5 ? 6 : nb == 10 ? 4 : 2; }
 
@@ -1548,7 +1550,7 @@ int launch_decode_merge(const DecodeArgs& a, int D, int B, cudaStream_t stream) 
     };
     e = nb == 5    ? go(std::integral_constant<int, 5>{})
         : nb == 10 ? go(std::integral_constant<int, 10>{})
-                   : go(std::integral_constant<int, 16>{});
+                   : go(std::integral_constant<int, 19>{});
   } else {
     if (a.span)
       e = (D == 256) ? cudaLaunchKernelEx(&mc, decode_merge_kernel<256, true>, a)

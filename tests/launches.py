@@ -1,4 +1,5 @@
-"""The kernel launches of a call, read from a stream capture (nothing runs)."""
+"""The kernel launches of a call, read from a stream capture (nothing runs), and a
+call's device time."""
 import ctypes
 from dataclasses import dataclass
 
@@ -70,3 +71,23 @@ def launches(call):
                             per_sm.value))
     do("cuGraphDestroy", graph)
     return found
+
+
+def device_us(call, calls=12, replays=20):
+    """Device time of ``call()`` among others of its kind, the median over replays of
+    a graph of them."""
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(calls):
+            call()
+    times = []
+    for _ in range(5 + replays):
+        start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        start.record()
+        graph.replay()
+        end.record()
+        end.synchronize()
+        times.append(start.elapsed_time(end) * 1e3 / calls)
+    return sorted(times[5:])[replays // 2]

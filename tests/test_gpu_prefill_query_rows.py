@@ -13,6 +13,7 @@ from oracle import attention as OT
 from paper_2609_17475_gb300 import synth
 from tests.cases import assert_attention_close, bits, make_case
 from tests.helpers import exact_groups, f64_to_bf16_tensor
+from tests.launches import device_us
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -46,7 +47,7 @@ def test_affine_prefill_large_query_rows(Hq, Hkv, D, q_start, C, big):
     assert_attention_close(out, ref)
 
 
-def _device_us(fmt, Hq, Hkv, D, C, calls=12):
+def _device_us(fmt, Hq, Hkv, D, C):
     codec = jf.Tq4Codec(D, [1] * D, [1] * D) if fmt == jf.JF_FMT_TQ4 else None
     pool = jf.KVPool.allocate(2, 64, Hkv, D, device=DEV, format=fmt, codec=codec)
     row = torch.zeros(2, dtype=torch.int32, device=DEV)
@@ -57,21 +58,7 @@ def _device_us(fmt, Hq, Hkv, D, C, calls=12):
     def call():
         jf.jf_prefill_chunk_attn(pool, row, q, 0, 0.1, True, out, ws)
 
-    call()
-    torch.cuda.synchronize()
-    graph = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(graph):
-        for _ in range(calls):
-            call()
-    times = []
-    for _ in range(20):
-        start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-        start.record()
-        graph.replay()
-        end.record()
-        end.synchronize()
-        times.append(start.elapsed_time(end) * 1e3 / calls)
-    return float(np.median(times[5:]))
+    return device_us(call)
 
 
 @pytest.mark.parametrize("fmt,C,bound", [(jf.JF_FMT_AFFINE4_G64, 8, 1.22), (jf.JF_FMT_TQ4, 20, 1.45)])
