@@ -58,8 +58,14 @@ __device__ __forceinline__ void two_sum_acc(float& sh, float& sl, float b) {
 // RN32(sqrt(s)) for the double-float sum s = sh + sl (error about 2^-40 s):
 // rounded from r = RN32(sqrt(sh)) and the exact residual sh - r^2 (one fma).
 // sure: the result is farther than 2^-10 half-ulp from a rounding boundary and
-// s is in the safe range.
+// s is in the safe range.  sl first leaves what sh can hold to sh: summed up, it
+// may be more than an ulp of it, r then more than one off, and the result not
+// sure (one vector in ~80 of the append's, each a wait for fp64: 9 rows of
+// 24/4/256, 5.2 us of device time, 2.8 now).
 __device__ __forceinline__ float rho_from_sum(float sh, float sl, bool& sure) {
+  const float hi = __fadd_rn(sh, sl);
+  sl = __fsub_rn(sl, __fsub_rn(hi, sh));                 // exact: |sl| <= |sh|
+  sh = hi;
   const float r = __fsqrt_rn(sh);
   const float res = __fmaf_rn(-r, r, sh);                // exact: s_hi - r^2
   // sqrt(s) = r + dl up to ~2^-41 r; rounding boundaries at half an ulp on
