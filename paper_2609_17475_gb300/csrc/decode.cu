@@ -1189,7 +1189,7 @@ __device__ __forceinline__ float ld_here(const float* p) {
 // the plan's splits: 38, 76 and 152 of them with four, two and one KV heads on 152
 // SMs (loads past the plan still cost their issue: ~0.1 us).  A second batch is
 // a second memory round trip: one request of 6/1/256 at 60,000 positions, 145 splits,
-// 12.5 us with batches of 16, 11.3 with 19.  Registers hold a batch, so an SM takes six, four or two CTAs.
+// 12.4 us with batches of 16, 11.2 with 19.  Registers hold a batch, so an SM takes six, four or two CTAs.
 constexpr int merge_nb(int rows) {
   return rows <= 5 * MERGE_NSG ? 5 : rows <= 10 * MERGE_NSG ? 10 : 19;
 }

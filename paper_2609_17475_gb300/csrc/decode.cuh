@@ -13,9 +13,10 @@ constexpr int DTOK = 32;      // positions per pipeline stage (one chunk)
 // fine, as far as the merge's rows allow.  Device time of a call with 16 / 12 /
 // 6 / 4 / 2 chunks: 1,000 positions (24/4/256) 10.2 / 8.5 / 7.4 / 7.1 / 7.2 us;
 // 4,096 (8/2/128) 7.5 / 6.7 / 5.9 / 5.8 / 6.0; a step at 8,000 10.3 / 9.0 / 8.2 /
-// 8.2 / 8.2; a verifier call at 1,000 15.4 / - / 10.1 / 9.1 / 8.4.  Two requests
-// of 700 and 1,500 positions with 16 / 8 / 6 / 4 places: 13.3 / 13.1 / 10.2 / 13.0
-// us (finer pieces hold only places of a request's start).
+// 8.2 / 8.2; a verifier call at 1,000 15.4 / - / 10.1 / 9.1 / 8.4.  Two requests of
+// 24/4/256, 21 pairs of 500 to 8,000 positions, on average with 4 / 6 / 8 / 12 / 16 /
+// 24 places: 12.1 / 12.1 / 12.5 / 12.7 / 13.3 / 14.6 us (one pair's own time moves by
+// up to 3 us from one value to the next, as a piece does or doesn't meet both).
 constexpr int MIN_CPS = 4;
 constexpr int SPAN_MIN = 6;
 constexpr float DTAU = 4.f;   // log2 headroom before the reference maximum moves
