@@ -1189,14 +1189,17 @@ __device__ __forceinline__ float ld_here(const float* p) {
 // the plan's splits: 38, 76 and 152 of them with four, two and one KV heads on 152
 // SMs (loads past the plan still cost their issue: ~0.1 us).  A second batch is
 // a second memory round trip: one request of 6/1/256 at 60,000 positions, 145 splits,
-// 12.4 us with batches of 16, 11.2 with 19.  Registers hold a batch, so an SM takes six, four or two CTAs.
+// 12.4 us with batches of 16, 11.2 with 19.  Registers hold a batch (40, 64 and 128
+// of them), so an SM takes six, four or two CTAs.  (Told so by the launch bounds
+// the compiler orders the kernel differently, with the same registers: a step at
+// 35,841 positions 15.4 -> 15.7 us.)
 constexpr int merge_nb(int rows) {
   return rows <= 5 * MERGE_NSG ? 5 : rows <= 10 * MERGE_NSG ? 10 : 19;
 }
 constexpr int merge_per_sm(int nb) { return nb == 5 ? 6 : nb == 10 ? 4 : 2; }
 
 template <int D, bool SPAN, int NB>
-__global__ void __launch_bounds__(MERGE_THREADS, merge_per_sm(NB)) decode_merge_sg_kernel(const DecodeArgs a) {
+__global__ void __launch_bounds__(MERGE_THREADS) decode_merge_sg_kernel(const DecodeArgs a) {
   // SPAN: partial rows of the span plan.  A template parameter: the span
   // branch in the single-request instance, though never taken, had slowed
   // the 256K call by ~1.2 us.
