@@ -358,6 +358,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     for (int i = threadIdx.x; i < 256 * 32; i += blockDim.x)
       lut[i] = pack_f16x2(a.cent[(i >> 5) & 15], a.cent[i >> 9]);
   }
+  // Instructions that a whole warp has to issue together (.aligned) come after a
+  // __syncwarp wherever a lane's own branch lies before them: nothing else is
+  // sure to bring the lanes back together.
+  __syncwarp();
   if (warp == 0) tc::alloc2(tmem_slot, 512);
   tc::fence_before();
   __syncthreads();
@@ -497,6 +501,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     __syncwarp();
     if (lane == 0) tc::arrive_cluster(q_full, 0);
   }
+  __syncwarp();
 
   if (warp < R::DQ0) {
   tc::setmaxnreg_dec<R::MMA_REGS>();
@@ -810,6 +815,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
       tc::fence_before();
       __syncwarp();
       if (lane == 0) tc::arrive_cluster(&p_full[j & 3], 0);
+      __syncwarp();
     }
     // epilogue: O / l -> bf16 (one split) or the unnormalized partial
     // (m, l, O) in fp32 (several), undoing the d order 0,4,1,5,2,6,3,7
@@ -893,6 +899,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
               *reinterpret_cast<uint4*>(orow + c0 + 8 * k) = w;
             }
           }
+          __syncwarp();
         }
       }
     } else {
@@ -904,6 +911,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
   // neither CTA may release TMEM or exit while its partner can still reach it
   tc::fence_before();
   __syncthreads();
+  __syncwarp();
   tc::cluster_sync();
   if (warp == 0) {
     tc::fence_after();
