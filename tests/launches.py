@@ -74,8 +74,8 @@ def launches(call):
 
 
 def device_us(call, calls=12, replays=20):
-    """Device time of ``call()`` among others of its kind, the median over replays of
-    a graph of them."""
+    """Device time of ``call()`` among others of its kind: the least over replays of a
+    graph of them (what else runs on the machine can only add to it)."""
     call()
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
@@ -90,4 +90,4 @@ def device_us(call, calls=12, replays=20):
         end.record()
         end.synchronize()
         times.append(start.elapsed_time(end) * 1e3 / calls)
-    return sorted(times[5:])[replays // 2]
+    return min(times[5:])
